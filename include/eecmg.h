@@ -423,9 +423,9 @@ eecmg_status eecmg_residual_noalloc(int width, int height, const double *psf, in
  * up to 16 blocks that exchange their sums through distributed shared memory
  * and stream the vectors through L2; larger levels run as a cooperative grid
  * of max(32x64 tiles, pixels / px_per_block) blocks, at most blocks_per_sm
- * per SM.  The fused start of a prolonged level runs on tiles of psd_tile_h
- * x 64 pixels (16 rows give small levels more blocks; its result does not
- * depend on the tile).  Process-wide.  Initial values: the GB300 optimum of
+ * per SM.  The fused start of a prolonged level runs in strip segments of at
+ * least psd_tile_h / 4 rows on levels that load the GPU (its result does not
+ * depend on them).  Process-wide.  Initial values: the GB300 optimum of
  * measured sweeps (resident_max_tiles 32, cluster_max_px 16384, px_per_block
  * 2048, blocks_per_sm 2, psd_tile_h 32), overridable by the environment
  * variables EECMG_RESIDENT_MAX_TILES, EECMG_CLUSTER_MAX_PX,
@@ -437,8 +437,8 @@ typedef struct {
     int px_per_block;         /* 1024 .. 4194304                              */
     int blocks_per_sm;        /* 1 .. 3                                       */
     int resident_max_tiles;   /* 0 .. 32; 0 = never shared-memory resident     */
-    int psd_tile_h;           /* 16 or 32: rows of the fused level start's
-                                 64-column tiles (Algorithm 2, Step 2)        */
+    int psd_tile_h;           /* 16 or 32: four times the least rows of the
+                                 fused level start's segments (Step 2)        */
 } eecmg_tuning;
 
 eecmg_status eecmg_get_tuning(eecmg_tuning *out);

@@ -116,15 +116,15 @@ void add_op(std::vector<OpGroup>& groups, size_t gi, int op, OpItem it) {
     if (groups.size() <= gi) groups.resize(gi + 1);
     groups[gi].op = op;
     it.bx = op_blocks_x(op, it.w);
-    if (op == OP_PSD) it.th = psd_tile_rows();
     groups[gi].items.push_back(it);
 }
 
 int place_items(OpGroup& g) {
     int blocks = 0;
+    if (g.op == OP_PSD) place_starts(g.items.data(), (int)g.items.size());
     for (auto& it : g.items) {
         it.block0 = blocks;
-        blocks += op_blocks(g.op, it.h, it.w);
+        blocks += op_blocks(g.op, it.h, it.w, it.th);
     }
     return blocks;
 }

@@ -94,11 +94,13 @@ struct OpItem {
     int h = 0, w = 0, h1 = 0, w1 = 0, h2 = 0, w2 = 0;
     float p0 = 0.f, p1 = 0.f, s0 = 0.f;
     int bx = 0, block0 = 0;
-    int th = 0;  // OP_PSD: rows of the item's tiles
+    int th = 0;  // OP_PSD: rows of the item's strip segments
 };
-int op_blocks(int op, int h, int w);  // blocks of operation kind op covering an h x w output
-int psd_tile_rows();                  // rows of the fused level start's tiles (process-wide tuning)
-int op_blocks_x(int op, int w);       // of which along x
+// blocks of operation kind op covering an h x w output (OP_PSD: in segments of th rows)
+int op_blocks(int op, int h, int w, int th = 0);
+int psd_tile_rows();                  // the level start's row parameter (process-wide tuning)
+int op_blocks_x(int op, int w);       // of which along x (OP_PSD: strips of columns)
+void place_starts(OpItem* items, int n);  // OP_PSD: sets th of the items of one launch
 cudaError_t launch_ops_batch(int op, const OpItem* d_items, int n, int total_blocks, cudaStream_t s);
 
 cudaError_t launch_restrict(const float* fine, int hf, int wf, float* coarse, int hc, int wc,

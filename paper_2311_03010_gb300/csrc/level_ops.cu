@@ -4,8 +4,11 @@
 // Eqs. 18-19) and one explicit Perona-Malik step D (Section 4, Eqs. 21-24).
 // Each runs once per level per restoration; they are simple stencils with
 // 32 x 8 thread blocks over the output image.
+#include <algorithm>
+
 #include "launch.hpp"
 #include "level_ops.cuh"
+#include "level_start.cuh"
 
 namespace eecmg {
 
@@ -193,17 +196,21 @@ __global__ void __launch_bounds__(BX* BY) k_denoise(const float* __restrict__ in
     tile_denoise(in, out, h, w, tau, inv_k2, blockIdx.y * BY, blockIdx.x * BX);
 }
 
-__global__ void __launch_bounds__(BX* BY) k_psd(const float* __restrict__ u1, int h1, int w1,
-                                               const float* __restrict__ u2, int h2, int w2,
-                                               float* __restrict__ out, int h, int w, float scale,
-                                               float tau, float inv_k2, int th) {
-    __shared__ PsdSmem M;
-    const int y0 = blockIdx.y * th, x0 = blockIdx.x * PSD_TW;
-    auto store = [&](int rr, int cc, float v) { out[(size_t)(y0 + rr) * w + x0 + cc] = v; };
-    if (th == 16)
-        tile_psd<16>(M, u1, h1, w1, u2, h2, w2, h, w, scale, tau, inv_k2, y0, x0, store);
-    else
-        tile_psd<PSD_TH>(M, u1, h1, w1, u2, h2, w2, h, w, scale, tau, inv_k2, y0, x0, store);
+__global__ void __launch_bounds__(32 * ST_WARPS, ST_MINB) k_psd(StartArgs a, int strips, int th) {
+    start_unit(a, strips, th, blockIdx.x * ST_WARPS + (threadIdx.x >> 5));
+}
+// The starts of many levels in one launch; items as in k_ops_batch (bx: strips).
+__global__ void __launch_bounds__(32 * ST_WARPS, ST_MINB) k_psd_batch(const OpItem* __restrict__ items, int n) {
+    const int blk = (int)blockIdx.x;
+    int lo = 0, hi = n - 1;
+    while (lo < hi) {
+        const int mid = (lo + hi + 1) >> 1;
+        if (items[mid].block0 <= blk) lo = mid;
+        else hi = mid - 1;
+    }
+    const OpItem& it = items[lo];
+    const StartArgs a{it.a, it.b, it.out, it.h1, it.w1, it.h2, it.w2, it.h, it.w, it.s0, it.p0, it.p1};
+    start_unit(a, it.bx, it.th, (blk - it.block0) * ST_WARPS + (threadIdx.x >> 5));
 }
 
 // Many operations of one kind in one launch (the server's ticks): block b
@@ -230,19 +237,6 @@ __global__ void __launch_bounds__(BX* BY) k_ops_batch(const OpItem* __restrict__
     if constexpr (OP == OP_DENOISE) tile_denoise(it.a, it.out, it.h, it.w, it.p0, it.p1, by * BY, bx * BX);
     if constexpr (OP == OP_PROLONG)
         tile_prolong(it.a, it.h1, it.w1, it.b, it.h2, it.w2, it.out, it.h, it.w, by * BY, bx * BX);
-    if constexpr (OP == OP_PSD) {
-        __shared__ PsdSmem M;
-        // this block's tile of the th x 64 grid (bx counts PSD_TW-wide tiles)
-        const int y0 = by * it.th, x0 = bx * PSD_TW;
-        float* out = it.out;
-        const int w = it.w;
-        auto store = [&](int rr, int cc, float v) { out[(size_t)(y0 + rr) * w + x0 + cc] = v; };
-        if (it.th == 16)
-            tile_psd<16>(M, it.a, it.h1, it.w1, it.b, it.h2, it.w2, it.h, it.w, it.s0, it.p0, it.p1, y0, x0, store);
-        else
-            tile_psd<PSD_TH>(M, it.a, it.h1, it.w1, it.b, it.h2, it.w2, it.h, it.w, it.s0, it.p0, it.p1, y0, x0,
-                             store);
-    }
     if constexpr (OP == OP_ZERO || OP == OP_COPY) {
         if (y < it.h && x < it.w) it.out[(size_t)y * it.w + x] = OP == OP_ZERO ? 0.f : it.a[(size_t)y * it.w + x];
     }
@@ -281,9 +275,12 @@ cudaError_t launch_prolong(const float* u1, int h1, int w1, const float* u2, int
 cudaError_t launch_psd(const float* u1, int h1, int w1, const float* u2, int h2, int w2, float* out,
                        int h, int w, float scale, float tau, float kpm, cudaStream_t s) {
     if (h <= 0 || w <= 0) return cudaSuccess;
-    const int th = psd_tile_rows();
-    const dim3 grid((w + PSD_TW - 1) / PSD_TW, (h + th - 1) / th);
-    k_psd<<<grid, dim3(BX, BY), 0, s>>>(u1, h1, w1, u2, h2, w2, out, h, w, scale, tau, 1.f / (kpm * kpm), th);
+    OpItem it;
+    it.h = h;
+    it.w = w;
+    place_starts(&it, 1);
+    const StartArgs a{u1, u2, out, h1, w1, h2, w2, h, w, scale, tau, 1.f / (kpm * kpm)};
+    k_psd<<<op_blocks(OP_PSD, h, w, it.th), 32 * ST_WARPS, 0, s>>>(a, op_blocks_x(OP_PSD, w), it.th);
     return cudaGetLastError();
 }
 
@@ -314,14 +311,38 @@ cudaError_t launch_denoise(const float* in, float* out, int h, int w, float tau,
     return cudaGetLastError();
 }
 
-int op_blocks(int op, int h, int w) {
+int op_blocks(int op, int h, int w, int th) {
     if (h <= 0 || w <= 0) return 0;
-    if (op == OP_PSD) return ((w + PSD_TW - 1) / PSD_TW) * ((h + psd_tile_rows() - 1) / psd_tile_rows());
+    if (op == OP_PSD) return (op_blocks_x(op, w) * ((h + th - 1) / th) + ST_WARPS - 1) / ST_WARPS;
     const dim3 g = grid2(h, w);
     return (int)(g.x * g.y);
 }
 
-int op_blocks_x(int op, int w) { return op == OP_PSD ? (w + PSD_TW - 1) / PSD_TW : (w + BX - 1) / BX; }
+int op_blocks_x(int op, int w) { return op == OP_PSD ? (w + ST_COLS - 1) / ST_COLS : (w + BX - 1) / BX; }
+
+// Rows per strip segment of the level starts of one launch (a segment computes
+// 6 rows more than it stores).  Where a quarter of the register file's warps
+// hold segments of MIN_ROWS, the chain of rows is the time: 9 us for a 64^2 to
+// 256^2 level in segments of 4 rows, 12 us in segments of 8.  Beyond that the
+// SMs are loaded and the extra rows count (1024^2: 17 us in 8 rows, 20 us in 4):
+// the fewest rows from psd_tile_rows() / 4 to 64 at which all segments are
+// resident at once.
+void place_starts(OpItem* items, int n) {
+    constexpr long long SMS = 152, MIN_ROWS = 4, MAX_ROWS = 64;
+    auto units = [&](long long th) {
+        long long u = 0;
+        for (int i = 0; i < n; ++i) u += (long long)op_blocks(OP_PSD, items[i].h, items[i].w, (int)th) * ST_WARPS;
+        return u;
+    };
+    long long th = MIN_ROWS;
+    if (units(th) > SMS * 5) {
+        const long long cap = SMS * ST_MINB * ST_WARPS;
+        const long long fit = units(1) / cap;
+        th = std::min(MAX_ROWS, std::max<long long>(psd_tile_rows() / 4, fit));
+        while (th < MAX_ROWS && units(th) > cap) ++th;
+    }
+    for (int i = 0; i < n; ++i) items[i].th = (int)th;
+}
 
 cudaError_t launch_ops_batch(int op, const OpItem* d_items, int n, int total_blocks, cudaStream_t s) {
     if (n <= 0 || total_blocks <= 0) return cudaSuccess;
@@ -335,7 +356,9 @@ cudaError_t launch_ops_batch(int op, const OpItem* d_items, int n, int total_blo
         case OP_ZERO: return launch_op<OP_ZERO>(d_items, n, total_blocks, s);
         case OP_COPY: return launch_op<OP_COPY>(d_items, n, total_blocks, s);
         case OP_PROLONG: return launch_op<OP_PROLONG>(d_items, n, total_blocks, s);
-        case OP_PSD: return launch_op<OP_PSD>(d_items, n, total_blocks, s);
+        case OP_PSD:
+            k_psd_batch<<<total_blocks, 32 * ST_WARPS, 0, s>>>(d_items, n);
+            return cudaGetLastError();
         default: return cudaErrorInvalidValue;
     }
 }

@@ -51,116 +51,145 @@ __device__ __forceinline__ float pi_at(const float* __restrict__ u1, int w1,
 static __constant__ float c_qw[4][3] = {
     {1.f, 0.f, 0.f}, {0.375f, 0.75f, -0.125f}, {0.f, 1.f, 0.f}, {-0.125f, 0.75f, 0.375f}};
 
+// MUFU approximations with subnormal results flushed (each about 1 ulp).  In
+// S a weight below 2^-126 adds nothing to sums of at least 1, the reciprocals'
+// arguments are kept away from zero, and no decision needs a correctly rounded
+// value (the eigenvalue cut at 1e-6 W lies where the dropped term is itself of
+// order 1e-6 of the neighbour differences).
+__device__ __forceinline__ float ex2_ftz(float x) {
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float rcp_ftz(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float sqrt_ftz(float x) {
+    float y;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
 // S: weighted least-squares plane fit over the in-image 3 x 3 neighbourhood
 // with weights exp(-(scale * (u_c - u_nb))^2) (Eqs. 18-19), output the fitted
 // constant.  Solved in centred form: with W, the weighted means (sb, tb, vb)
 // of the offsets and of v = u_nb - u_c, the 2 x 2 moment matrix C and the
 // cross vector c, slope = C^+ c (eigenvalues below 1e-6 W dropped) and
 // a0 = u_c + vb - slope . (sb, tb).
-// EDGE = false: the caller guarantees that the whole 3 x 3 neighbourhood lies in
-// the image (the same arithmetic without the bounds tests).
+// The arithmetic is written as two pieces that every kernel shares, with the
+// rounding of each operation fixed (no contraction), so that the kernels'
+// results agree bitwise: the pair terms below, and s_value.
+
+// exp(-(scale v)^2) from ks = scale sqrt(log2 e): the weight of a pair of
+// neighbours; it does not depend on which of the two is the centre.
+__device__ __forceinline__ float s_scale_ks(float scale) { return __fmul_rn(scale, 1.2011224087864498f); }
+__device__ __forceinline__ float s_weight(float v, float ks) {
+    const float t = __fmul_rn(v, ks);
+    return ex2_ftz(__fmul_rn(t, -t));
+}
+// One row of three neighbours (columns -1, 0, 1): weights l, c, r, the
+// products weight x v, and their sums.
+struct SRow {
+    float l, r, sum;     // the centre column enters through the sum only
+    float lv, rv, sumv;
+};
+__device__ __forceinline__ SRow s_row(float l, float c, float r, float lv, float cv, float rv) {
+    return SRow{l, r, __fadd_rn(__fadd_rn(l, c), r), lv, rv, __fadd_rn(__fadd_rn(lv, cv), rv)};
+}
+// S's value from the row above (s = -1), the row below (s = 1) and the two
+// neighbours in the centre's own row (weights d, f, products dv, fv).  The
+// moments are taken raw and centred afterwards: offsets are in {-1, 0, 1}
+// and the centre has weight 1, so a centred diagonal moment is at least 1/9 of
+// the raw one and the subtraction costs no more than the centred sums did.
+__device__ __forceinline__ float s_value(float uc, const SRow& N, const SRow& P, float d, float f, float dv,
+                                         float fv) {
+    const float mss = __fadd_rn(N.sum, P.sum), sb = __fadd_rn(P.sum, -N.sum);
+    const float cm = __fadd_rn(__fadd_rn(N.l, d), P.l), cp = __fadd_rn(__fadd_rn(N.r, f), P.r);
+    const float mtt = __fadd_rn(cm, cp), tb = __fadd_rn(cp, -cm);
+    const float mst = __fadd_rn(__fadd_rn(N.l, P.r), -__fadd_rn(N.r, P.l));
+    const float W = __fadd_rn(__fadd_rn(__fadd_rn(d, f), mss), 1.f);
+    const float rsv = __fadd_rn(P.sumv, -N.sumv);
+    const float cvm = __fadd_rn(__fadd_rn(N.lv, dv), P.lv), cvp = __fadd_rn(__fadd_rn(N.rv, fv), P.rv);
+    const float rtv = __fadd_rn(cvp, -cvm);
+    const float sv = __fadd_rn(__fadd_rn(N.sumv, P.sumv), __fadd_rn(dv, fv));
+    const float iw = rcp_ftz(W);  // 1 <= W <= 9
+    const float so = __fmul_rn(sb, iw), to = __fmul_rn(tb, iw), vb = __fmul_rn(sv, iw);
+    const float css = __fmaf_rn(-so, sb, mss), cst = __fmaf_rn(-so, tb, mst), ctt = __fmaf_rn(-to, tb, mtt);
+    const float csv = __fmaf_rn(-vb, sb, rsv), ctv = __fmaf_rn(-vb, tb, rtv);
+    // eigenvalues l1 >= l2 (the small one from the determinant: no
+    // cancellation), an unnormalised eigenvector (es, et) of l1 from the row of
+    // C - l2 I with the larger diagonal, and (-et, es) of l2
+    const float tr = __fmul_rn(0.5f, __fadd_rn(css, ctt)), df = __fmul_rn(0.5f, __fadd_rn(css, -ctt));
+    const float l1 = __fadd_rn(tr, sqrt_ftz(__fmaf_rn(df, df, __fmul_rn(cst, cst))));
+    const float r1 = rcp_ftz(l1);
+    const float l2 = __fmul_rn(__fmaf_rn(css, ctt, -__fmul_rn(cst, cst)), r1);
+    const float thr = __fmul_rn(1e-6f, W);
+    const float a0 = __fadd_rn(css, -l2), c0 = __fadd_rn(ctt, -l2);
+    const bool big = fabsf(a0) >= fabsf(c0);
+    float es = big ? a0 : cst, et = big ? cst : c0;
+    float nn = __fmaf_rn(es, es, __fmul_rn(et, et));
+    if (!(nn > 0.f)) {  // C = l1 I: any pair of axes
+        es = 1.f;
+        et = 0.f;
+        nn = 1.f;
+    }
+    // slope . ob = [ (e1.c)(e1.ob) / l1 + (e2.c)(e2.ob) / l2 ] / |e|^2
+    const float p1 = __fmul_rn(__fmaf_rn(es, csv, __fmul_rn(et, ctv)), __fmaf_rn(es, so, __fmul_rn(et, to)));
+    const float p2 = __fmul_rn(__fmaf_rn(es, ctv, -__fmul_rn(et, csv)), __fmaf_rn(es, to, -__fmul_rn(et, so)));
+    const float t2 = l2 > thr ? __fmul_rn(p2, rcp_ftz(l2)) : 0.f;
+    const float g = __fmul_rn(__fmaf_rn(p1, r1, t2), rcp_ftz(nn));
+    return __fadd_rn(__fadd_rn(uc, vb), l1 > thr ? -g : 0.f);
+}
+// S at one pixel from a reader of the image; EDGE = false: the caller guarantees
+// that the whole 3 x 3 neighbourhood lies in the image (no bounds tests).
 template <bool EDGE = true, class Rd>
 __device__ __forceinline__ float smooth_value_rd(Rd rd, int h, int w, float scale, int i, int j) {
-    const float uc = rd(i, j);
-    float ws[9], ss[9], ts[9], vs[9];
-    float W = 0.f, sb = 0.f, tb = 0.f, vb = 0.f;
-#pragma unroll
-    for (int s = -1; s <= 1; ++s) {
-#pragma unroll
-        for (int t = -1; t <= 1; ++t) {
-            const int k = (s + 1) * 3 + (t + 1);
-            const int ii = i + s, jj = j + t;
-            const bool inside = !EDGE || (ii >= 0 && ii < h && jj >= 0 && jj < w);
-            // the centre term is v = 0, weight exp(0) = 1 exactly (as the exponential gives it)
-            const bool ctr = s == 0 && t == 0;
-            const float v = ctr ? 0.f : (inside ? rd(ii, jj) - uc : 0.f);
-            const float e = scale * v;
-            const float wt = ctr ? 1.f : (inside ? __expf(-e * e) : 0.f);  // MUFU exp: ~2 ulp, ample for a weight
-            ws[k] = wt;
-            ss[k] = (float)s;
-            ts[k] = (float)t;
-            vs[k] = v;
-            W += wt;
-            // a zero offset (or the centre's v = 0) adds exactly nothing: no FMA for it
-            if (s != 0) sb = fmaf(wt, (float)s, sb);
-            if (t != 0) tb = fmaf(wt, (float)t, tb);
-            if (!ctr) vb = fmaf(wt, v, vb);
-        }
-    }
-    const float inv_w = 1.f / W;  // W >= 1: the centre always has weight 1
-    sb *= inv_w;
-    tb *= inv_w;
-    vb *= inv_w;
-    float css = 0.f, cst = 0.f, ctt = 0.f, csv = 0.f, ctv = 0.f;
+    const float uc = rd(i, j), ks = s_scale_ks(scale);
+    float wt[9], wv[9];
 #pragma unroll
     for (int k = 0; k < 9; ++k) {
-        const float ds = ss[k] - sb, dt = ts[k] - tb, dv = vs[k] - vb;
-        const float wd = ws[k];
-        css = fmaf(wd * ds, ds, css);
-        cst = fmaf(wd * ds, dt, cst);
-        ctt = fmaf(wd * dt, dt, ctt);
-        csv = fmaf(wd * ds, dv, csv);
-        ctv = fmaf(wd * dt, dv, ctv);
+        const int ii = i + k / 3 - 1, jj = j + k % 3 - 1;
+        const bool inside = k != 4 && (!EDGE || (ii >= 0 && ii < h && jj >= 0 && jj < w));
+        const float v = inside ? __fadd_rn(rd(ii, jj), -uc) : 0.f;
+        wt[k] = inside ? s_weight(v, ks) : 0.f;
+        wv[k] = __fmul_rn(wt[k], v);
     }
-    const float tr = 0.5f * (css + ctt), df = 0.5f * (css - ctt);
-    const float rad = sqrtf(df * df + cst * cst);
-    const float l1 = tr + rad;
-    // small eigenvalue from the determinant: no cancellation
-    const float l2 = l1 > 0.f ? (css * ctt - cst * cst) / l1 : 0.f;
-    const float thr = 1e-6f * W;
-    float e1s = 1.f, e1t = 0.f;
-    if (rad > 0.f) {
-        const float a0 = css - l2, c0 = ctt - l2;
-        if (fabsf(a0) >= fabsf(c0)) {
-            const float nn = rsqrtf(a0 * a0 + cst * cst);
-            e1s = a0 * nn;
-            e1t = cst * nn;
-        } else {
-            const float nn = rsqrtf(cst * cst + c0 * c0);
-            e1s = cst * nn;
-            e1t = c0 * nn;
-        }
-    }
-    const float e2s = -e1t, e2t = e1s;
-    // the slope's components along the eigenvectors: no decision depends on them, so the
-    // fast division (2 ulp) serves; the eigenvalues, which the cut tests, stay IEEE-rounded
-    float gs = 0.f, gt = 0.f;
-    if (l1 > thr) {
-        const float c1 = __fdividef(e1s * csv + e1t * ctv, l1);
-        gs = fmaf(c1, e1s, gs);
-        gt = fmaf(c1, e1t, gt);
-    }
-    if (l2 > thr) {
-        const float c2 = __fdividef(e2s * csv + e2t * ctv, l2);
-        gs = fmaf(c2, e2s, gs);
-        gt = fmaf(c2, e2t, gt);
-    }
-    return uc + vb - (gs * sb + gt * tb);
+    return s_value(uc, s_row(wt[0], wt[1], wt[2], wv[0], wv[1], wv[2]),
+                   s_row(wt[6], wt[7], wt[8], wv[6], wv[7], wv[8]), wt[3], wt[5], wv[3], wv[5]);
 }
+
 // D: u + tau * sum over in-image 4-neighbours of (c_nb + c_c)/2 (u_nb - u_c),
 // c = 1 / (1 + |grad u|^2 / k^2) with central differences (an out-of-image
 // neighbour replaced by the centre value).
+__device__ __forceinline__ float pm_c_value(float ue, float uw, float us, float un, float inv_k2) {
+    const float gx = __fmul_rn(0.5f, __fadd_rn(ue, -uw)), gy = __fmul_rn(0.5f, __fadd_rn(us, -un));
+    return rcp_ftz(__fmaf_rn(__fmaf_rn(gx, gx, __fmul_rn(gy, gy)), inv_k2, 1.f));
+}
+// the flux from b into a (the flux from a into b is its negative)
+__device__ __forceinline__ float pm_flux(float ca, float cb, float ua, float ub) {
+    return __fmul_rn(__fmul_rn(0.5f, __fadd_rn(ca, cb)), __fadd_rn(ub, -ua));
+}
+// the step from the four fluxes (0 for a neighbour outside the image)
+__device__ __forceinline__ float pm_step(float uc, float fe, float fw, float fn, float fs, float tau) {
+    return __fmaf_rn(tau, __fadd_rn(__fadd_rn(__fadd_rn(fe, fw), fn), fs), uc);
+}
 template <class Rd>
 __device__ __forceinline__ float pm_c_rd(Rd u, int h, int w, int i, int j, float inv_k2) {
     const float uc = u(i, j);
-    const float ue = (j + 1 < w) ? u(i, j + 1) : uc;
-    const float uw = (j > 0) ? u(i, j - 1) : uc;
-    const float us = (i + 1 < h) ? u(i + 1, j) : uc;
-    const float un = (i > 0) ? u(i - 1, j) : uc;
-    const float gx = 0.5f * (ue - uw), gy = 0.5f * (us - un);
-    return 1.f / (1.f + (gx * gx + gy * gy) * inv_k2);
+    return pm_c_value((j + 1 < w) ? u(i, j + 1) : uc, (j > 0) ? u(i, j - 1) : uc, (i + 1 < h) ? u(i + 1, j) : uc,
+                      (i > 0) ? u(i - 1, j) : uc, inv_k2);
 }
 // c at (i, j) from a reader Cd of precomputed c, u from Ud.
 template <class Ud, class Cd>
 __device__ __forceinline__ float denoise_value_rd(Ud in, Cd c, int h, int w, float tau, int i, int j) {
-    const float uc = in(i, j);
-    const float cc = c(i, j);
-    float f = 0.f;
-    if (i + 1 < h) f += 0.5f * (c(i + 1, j) + cc) * (in(i + 1, j) - uc);
-    if (i > 0) f += 0.5f * (c(i - 1, j) + cc) * (in(i - 1, j) - uc);
-    if (j + 1 < w) f += 0.5f * (c(i, j + 1) + cc) * (in(i, j + 1) - uc);
-    if (j > 0) f += 0.5f * (c(i, j - 1) + cc) * (in(i, j - 1) - uc);
-    return fmaf(tau, f, uc);
+    const float uc = in(i, j), cc = c(i, j);
+    const float fe = j + 1 < w ? pm_flux(cc, c(i, j + 1), uc, in(i, j + 1)) : 0.f;
+    const float fw = j > 0 ? pm_flux(cc, c(i, j - 1), uc, in(i, j - 1)) : 0.f;
+    const float fn = i > 0 ? pm_flux(cc, c(i - 1, j), uc, in(i - 1, j)) : 0.f;
+    const float fs = i + 1 < h ? pm_flux(cc, c(i + 1, j), uc, in(i + 1, j)) : 0.f;
+    return pm_step(uc, fe, fw, fn, fs, tau);
 }
 // The start of a prolonged level (Algorithm 2, Step 2) in one pass: D(S(P(Pi(u1, u2)))) for
 // one TH x PSD_TW block of fine pixels at (y0, x0), TH <= PSD_TH (the shared-memory stages are
