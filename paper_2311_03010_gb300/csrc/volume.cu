@@ -23,13 +23,10 @@
 // the grid barrier with the fused deterministic reduction of persistent.cuh
 // (every block sums all blocks' partials in a fixed order and keeps its own
 // replica of the scalars), so the m_l iterations never return to the host and
-// the stop decision is taken on the device.  The convolution phases loop over
-// 8 x 8 x 32 output tiles: a tile and its halo are staged in shared memory and
-// a separable PSF runs as three passes (slices, rows, columns) inside the tile;
-// a general PSF runs its non-zero taps from the staged tile (the level solve is
-// in volume_impl.cuh).  The level start (Pi, P, S, D) is a chain of
-// voxel-parallel kernels in this file.  The cascade is captured once as a CUDA
-// graph.
+// the stop decision is taken on the device.  The convolution phases march tiles
+// of columns along the slices from a ring of staged planes (the level solve is in
+// volume_impl.cuh).  The level start (Pi, P, S, D) is a chain of kernels in
+// volume_start.cu.  The cascade is captured once as a CUDA graph.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -38,6 +35,7 @@
 
 #include "plan.hpp"
 #include "volume_impl.cuh"
+#include "volume_start.hpp"
 
 namespace eecmg {
 namespace vol {
@@ -57,210 +55,6 @@ __global__ void __launch_bounds__(VBX * VBY) k_vol_restrict(const float* __restr
                                                             float* __restrict__ c, int dc, int hc, int wc) {
     VOXEL_INDEX(dc, hc, wc)
     c[v] = f[((long long)(2 * k) * hf + 2 * i) * wf + 2 * j];
-}
-
-// Pi: out = u1 + (1/4) * mean of the level-(l-2) differences d over the cell's
-// eight corners (indices past the last level-(l-2) node clamp to it).
-__global__ void __launch_bounds__(VBX * VBY) k_vol_pi(const float* __restrict__ u1, int d1, int h1, int w1,
-                                                      const float* __restrict__ u2, int d2, int h2, int w2,
-                                                      float* __restrict__ out) {
-    VOXEL_INDEX(d1, h1, w1)
-    const int c = k, a = i, b = j;
-    const int C0 = c >> 1, C1 = (c & 1) ? min(C0 + 1, d2 - 1) : C0;
-    const int A0 = a >> 1, A1 = (a & 1) ? min(A0 + 1, h2 - 1) : A0;
-    const int B0 = b >> 1, B1 = (b & 1) ? min(B0 + 1, w2 - 1) : B0;
-    const int Cs[2] = {C0, C1}, As[2] = {A0, A1}, Bs[2] = {B0, B1};
-    float s = 0.f;
-#pragma unroll
-    for (int x = 0; x < 2; ++x)
-#pragma unroll
-        for (int y = 0; y < 2; ++y)
-#pragma unroll
-            for (int z = 0; z < 2; ++z)
-                s += __ldg(u1 + ((long long)(2 * Cs[x]) * h1 + 2 * As[y]) * w1 + 2 * Bs[z]) -
-                     __ldg(u2 + ((long long)Cs[x] * h2 + As[y]) * w2 + Bs[z]);
-    out[v] = u1[v] + 0.03125f * s;
-}
-
-__constant__ float c_vqw[4][3] = {
-    {1.f, 0.f, 0.f}, {0.375f, 0.75f, -0.125f}, {0.f, 1.f, 0.f}, {-0.125f, 0.75f, 0.375f}};
-
-// P: the three-point quadratic rule along all three axes (clamped indices).
-__global__ void __launch_bounds__(VBX * VBY) k_vol_quad(const float* __restrict__ ut, int d1, int h1, int w1,
-                                                        float* __restrict__ out, int d, int h, int w) {
-    VOXEL_INDEX(d, h, w)
-    const int tz = k & 3, ty = i & 3, tx = j & 3;
-    const int Z = (k >> 2) * 2, Y = (i >> 2) * 2, X = (j >> 2) * 2;
-    int xs[3];
-#pragma unroll
-    for (int q = 0; q < 3; ++q) xs[q] = min(X + q, w1 - 1);
-    float s = 0.f;
-#pragma unroll
-    for (int o = 0; o < 3; ++o) {
-        const float wz = c_vqw[tz][o];
-        if (wz == 0.f) continue;
-        const int c = min(Z + o, d1 - 1);
-        float sy = 0.f;
-#pragma unroll
-        for (int p = 0; p < 3; ++p) {
-            const float wy = c_vqw[ty][p];
-            if (wy == 0.f) continue;
-            const float* row = ut + ((long long)c * h1 + min(Y + p, h1 - 1)) * w1;
-            float sx = 0.f;
-#pragma unroll
-            for (int q = 0; q < 3; ++q) sx = fmaf(c_vqw[tx][q], __ldg(row + xs[q]), sx);
-            sy = fmaf(wy, sx, sy);
-        }
-        s = fmaf(wz, sy, s);
-    }
-    out[v] = s;
-}
-
-// slope . ob for slope = C^+ c (eigenvalues of C at most thr dropped), by the
-// cyclic Jacobi method (Golub & Van Loan, Sec. 8.5): rotations in the (0,1),
-// (0,2), (1,2) planes diagonalise the symmetric C; instead of accumulating
-// the eigenvector matrix V, each rotation is applied to c and ob directly, so
-// y = V^T c and z = V^T ob and the result is sum_k [lambda_k > thr] y_k z_k /
-// lambda_k.  A rotation's angle needs no correct rounding (the rotation stays
-// orthogonal to rounding whatever its angle, and the next sweep removes what
-// it left), so t uses the fast division (its denominator is at least 1).
-// Four sweeps.
-__device__ __forceinline__ float jacobi_pinv_dot(float (&A)[3][3], float (&y)[3], float (&z)[3],
-                                                 float thr) {
-#pragma unroll
-    for (int sweep = 0; sweep < 4; ++sweep) {
-#pragma unroll
-        for (int pq = 0; pq < 3; ++pq) {
-            const int p = pq == 2 ? 1 : 0, q = pq == 0 ? 1 : 2, r = 3 - p - q;
-            const float apq = A[p][q];
-            if (apq == 0.f) continue;
-            const float th = (A[q][q] - A[p][p]) / (2.f * apq);  // IEEE: apq may be subnormal
-            const float t = __fdividef(copysignf(1.f, th), fabsf(th) + sqrtf(fmaf(th, th, 1.f)));
-            const float c = rsqrtf(fmaf(t, t, 1.f)), s = t * c;
-            A[p][p] = fmaf(-t, apq, A[p][p]);
-            A[q][q] = fmaf(t, apq, A[q][q]);
-            A[p][q] = A[q][p] = 0.f;
-            const float arp = A[r][p], arq = A[r][q];
-            A[r][p] = A[p][r] = c * arp - s * arq;
-            A[r][q] = A[q][r] = s * arp + c * arq;
-            const float yp = y[p], yq = y[q], zp = z[p], zq = z[q];
-            y[p] = c * yp - s * yq;
-            y[q] = s * yp + c * yq;
-            z[p] = c * zp - s * zq;
-            z[q] = s * zp + c * zq;
-        }
-    }
-    float g = 0.f;
-#pragma unroll
-    for (int k = 0; k < 3; ++k)
-        if (A[k][k] > thr) g = fmaf(__fdividef(y[k], A[k][k]), z[k], g);
-    return g;
-}
-
-// S: per voxel, the weighted hyperplane fit over the in-volume 3x3x3
-// neighbourhood (weights exp(-(scale v)^2), v = neighbour - centre) in centred
-// form; the output is u + vb - slope . ob with slope = C^+ c.  When
-// Gershgorin's bound puts every eigenvalue of C above 1e-2 W (far above the
-// 1e-6 W cut), C^+ = C^-1 and the slope comes from the adjugate; otherwise from
-// the Jacobi eigen-decomposition with the cut.
-__global__ void __launch_bounds__(VBX * VBY) k_vol_smooth(const float* __restrict__ u, int d, int h, int w,
-                                                          float scale, float* __restrict__ out) {
-    VOXEL_INDEX(d, h, w)
-    const float uc = u[v];
-    float W = 0.f, o0 = 0.f, o1 = 0.f, o2 = 0.f, vb = 0.f;
-    float m00 = 0.f, m01 = 0.f, m02 = 0.f, m11 = 0.f, m12 = 0.f, m22 = 0.f;
-    float c0 = 0.f, c1 = 0.f, c2 = 0.f;
-    // raw weighted moments; centred afterwards (offsets are small integers)
-#pragma unroll
-    for (int r = -1; r <= 1; ++r) {
-        if (k + r < 0 || k + r >= d) continue;
-#pragma unroll
-        for (int s = -1; s <= 1; ++s) {
-            if (i + s < 0 || i + s >= h) continue;
-            const float* row = u + ((long long)(k + r) * h + i + s) * w + j;
-#pragma unroll
-            for (int t = -1; t <= 1; ++t) {
-                if (j + t < 0 || j + t >= w) continue;
-                const float val = __ldg(row + t) - uc;
-                const float e = scale * val;
-                const float wt = (r == 0 && s == 0 && t == 0) ? 1.f : __expf(-e * e);
-                W += wt;
-                const float wv = wt * val;
-                vb += wv;
-                if (r) { o0 = fmaf(wt, (float)r, o0); m00 += wt; c0 = fmaf(wv, (float)r, c0); }
-                if (s) { o1 = fmaf(wt, (float)s, o1); m11 += wt; c1 = fmaf(wv, (float)s, c1); }
-                if (t) { o2 = fmaf(wt, (float)t, o2); m22 += wt; c2 = fmaf(wv, (float)t, c2); }
-                if (r && s) m01 = fmaf(wt, (float)(r * s), m01);
-                if (r && t) m02 = fmaf(wt, (float)(r * t), m02);
-                if (s && t) m12 = fmaf(wt, (float)(s * t), m12);
-            }
-        }
-    }
-    const float iW = 1.f / W;
-    o0 *= iW; o1 *= iW; o2 *= iW; vb *= iW;
-    // centred moments: sum w (o - ob)(o' - ob') = sum w o o' - W ob ob'
-    float A[3][3];
-    A[0][0] = fmaf(-W * o0, o0, m00);
-    A[1][1] = fmaf(-W * o1, o1, m11);
-    A[2][2] = fmaf(-W * o2, o2, m22);
-    A[0][1] = A[1][0] = fmaf(-W * o0, o1, m01);
-    A[0][2] = A[2][0] = fmaf(-W * o0, o2, m02);
-    A[1][2] = A[2][1] = fmaf(-W * o1, o2, m12);
-    // sum w (o - ob)(v - vb) = sum w o v - W ob vb
-    const float cv0 = fmaf(-W * o0, vb, c0), cv1 = fmaf(-W * o1, vb, c1), cv2 = fmaf(-W * o2, vb, c2);
-    const float gersh = fminf(A[0][0] - fabsf(A[0][1]) - fabsf(A[0][2]),
-                              fminf(A[1][1] - fabsf(A[0][1]) - fabsf(A[1][2]),
-                                    A[2][2] - fabsf(A[0][2]) - fabsf(A[1][2])));
-    float gob;
-    if (gersh > 1e-2f * W) {
-        const float k00 = A[1][1] * A[2][2] - A[1][2] * A[1][2];
-        const float k01 = A[0][2] * A[1][2] - A[0][1] * A[2][2];
-        const float k02 = A[0][1] * A[1][2] - A[0][2] * A[1][1];
-        const float k11 = A[0][0] * A[2][2] - A[0][2] * A[0][2];
-        const float k12 = A[0][1] * A[0][2] - A[0][0] * A[1][2];
-        const float k22 = A[0][0] * A[1][1] - A[0][1] * A[0][1];
-        const float idet = 1.f / (A[0][0] * k00 + A[0][1] * k01 + A[0][2] * k02);
-        const float g0 = (k00 * cv0 + k01 * cv1 + k02 * cv2) * idet;
-        const float g1 = (k01 * cv0 + k11 * cv1 + k12 * cv2) * idet;
-        const float g2 = (k02 * cv0 + k12 * cv1 + k22 * cv2) * idet;
-        gob = g0 * o0 + g1 * o1 + g2 * o2;
-    } else {
-        float y[3] = {cv0, cv1, cv2}, z[3] = {o0, o1, o2};
-        gob = jacobi_pinv_dot(A, y, z, 1e-6f * W);
-    }
-    out[v] = uc + vb - gob;
-}
-
-// D, first half: the diffusivity c = 1 / (1 + |grad u|^2 / k^2), central
-// differences, an out-of-volume neighbour replaced by the centre.
-__global__ void __launch_bounds__(VBX * VBY) k_vol_pm_c(const float* __restrict__ u, int d, int h, int w,
-                                                        float ik2, float* __restrict__ c) {
-    VOXEL_INDEX(d, h, w)
-    const long long sl = (long long)h * w;
-    const float uc = u[v];
-    const float ub = k + 1 < d ? u[v + sl] : uc, ua = k > 0 ? u[v - sl] : uc;
-    const float us = i + 1 < h ? u[v + w] : uc, un = i > 0 ? u[v - w] : uc;
-    const float ue = j + 1 < w ? u[v + 1] : uc, uw = j > 0 ? u[v - 1] : uc;
-    const float gx = 0.5f * (ue - uw), gy = 0.5f * (us - un), gz = 0.5f * (ub - ua);
-    c[v] = 1.f / (1.f + (gx * gx + gy * gy + gz * gz) * ik2);
-}
-
-// D, second half: u' = u + tau sum over in-volume face neighbours of
-// (c_nb + c) / 2 (u_nb - u) (no flux through the volume's faces).
-__global__ void __launch_bounds__(VBX * VBY) k_vol_pm_step(const float* __restrict__ u, const float* __restrict__ c,
-                                                           int d, int h, int w, float tau,
-                                                           float* __restrict__ out) {
-    VOXEL_INDEX(d, h, w)
-    const long long sl = (long long)h * w;
-    const float uc = u[v], cc = c[v];
-    float f = 0.f;
-    if (k + 1 < d) f = fmaf(0.5f * (c[v + sl] + cc), u[v + sl] - uc, f);
-    if (k > 0) f = fmaf(0.5f * (c[v - sl] + cc), u[v - sl] - uc, f);
-    if (i + 1 < h) f = fmaf(0.5f * (c[v + w] + cc), u[v + w] - uc, f);
-    if (i > 0) f = fmaf(0.5f * (c[v - w] + cc), u[v - w] - uc, f);
-    if (j + 1 < w) f = fmaf(0.5f * (c[v + 1] + cc), u[v + 1] - uc, f);
-    if (j > 0) f = fmaf(0.5f * (c[v - 1] + cc), u[v - 1] - uc, f);
-    out[v] = fmaf(tau, f, uc);
 }
 
 }  // namespace vol
@@ -354,7 +148,6 @@ void make_vol_taps(const std::vector<double>& K, int kd, int kh, int kw, bool tr
             for (int q = 0; q < kw; ++q) t->cx[q - rx + r] = (float)c[q];
         }
     }
-    t->sep = sep ? 1 : 0;
     list->clear();
     if (!sep) {
         for (int o = -rz; o <= rz; ++o)
@@ -370,13 +163,30 @@ void make_vol_taps(const std::vector<double>& K, int kd, int kh, int kw, bool tr
                 }
     }
     t->ntap = (int)list->size();
+    // Rows of 2 r + 1 taps cost (2 r + 1) multiplications per row that holds a tap, on
+    // register windows; a list costs a shared-memory read and a tap fetch per tap.  Up to
+    // four times the multiplications the rows win (5^3 full support, 96 x 121 x 150: 13 us a
+    // convolution against 157 us for the list).
+    std::vector<char> row((size_t)kd * kh, 0);
+    for (const int4& e : *list) row[(size_t)(e.x + rz) * kh + (e.y + ry)] = 1;
+    const int rows = (int)std::count(row.begin(), row.end(), 1);
+    t->form = sep ? VF_SEP : (rows * (2 * r + 1) <= 4 * t->ntap ? VF_DENSE : VF_SPARSE);
 }
 
 size_t align256(size_t x) { return (x + 255) & ~(size_t)255; }
 
-size_t tile_bytes(const VolTaps& t) {
-    const int NZ = TZ + 2 * t.r, NY = TY + 2 * t.r, AX = TX + 2 * ((t.r + 3) / 4 * 4);
-    return sizeof(float) * (2 * (size_t)NZ * NY * AX + (t.sep ? (size_t)TZ * NY * AX : 0));
+// Shared memory and tile rows of the kernels of radius r applying a PSF in `form`.
+template <int R = VR>
+size_t form_bytes(int r, int form) {
+    if constexpr (R > 0)
+        if (r < R) return form_bytes<R - 1>(r, form);
+    return vol_smem<R>(form);
+}
+template <int R = VR>
+int form_rows(int r, int form) {
+    if constexpr (R > 0)
+        if (r < R) return form_rows<R - 1>(r, form);
+    return vol_tile_rows<R>(form);
 }
 
 // The kernels of every radius 0 .. EECMG_VOL_MAX_RADIUS (instantiated in the
@@ -430,15 +240,17 @@ VolJob make_job(eecmg_vol_s* P, int l, bool transpose) {
     return J;
 }
 
-int level_tiles(const VolJob& J) {
-    return ((J.w + TX - 1) / TX) * ((J.h + TY - 1) / TY) * ((J.d + TZ - 1) / TZ);
+// The (tile, slice) pairs a convolution phase divides over the blocks.
+long long level_units(int d, int h, int w, const VolTaps& t) {
+    const int sy = form_rows(t.r, t.form);
+    return (long long)((w + MX - 1) / MX) * ((h + sy - 1) / sy) * d;
 }
 
 eecmg_status launch_solve(eecmg_vol_s* P, int l, bool zero_start, cudaStream_t s) {
     VolJob J = make_job(P, l, false);
     J.zero_start = zero_start ? 1 : 0;
     void* args[] = {&J};
-    const size_t smem = tile_bytes(J.taps);
+    const size_t smem = form_bytes(J.taps.r, J.taps.form);
     VCK(cudaLaunchCooperativeKernel(vol_kernels().solve[J.taps.r], dim3(P->grid[l]), dim3(NTHREADS),
                                     args, smem, s));
     return EECMG_OK;
@@ -447,11 +259,11 @@ eecmg_status launch_solve(eecmg_vol_s* P, int l, bool zero_start, cudaStream_t s
 eecmg_status launch_apply(eecmg_vol_s* P, int l, bool transpose, const float* x, float* y,
                           cudaStream_t s) {
     VolJob J = make_job(P, l, transpose);
-    const size_t smem = tile_bytes(J.taps);
+    const size_t smem = form_bytes(J.taps.r, J.taps.form);
     const float* xx = x;
     void* args[] = {&J, (void*)&xx, (void*)&y};
-    VCK(cudaLaunchKernel(vol_kernels().apply[J.taps.r], dim3(level_tiles(J)), dim3(NTHREADS), args,
-                         smem, s));
+    VCK(cudaLaunchKernel(vol_kernels().apply[J.taps.r], dim3((unsigned int)std::min<long long>(level_units(J.d, J.h, J.w, J.taps), 2 * P->sms)), dim3(NTHREADS),
+                         args, smem, s));
     return EECMG_OK;
 }
 
@@ -465,20 +277,17 @@ eecmg_status launch_start(eecmg_vol_s* P, int l, const float* u1, const float* u
     float* ut = P->vec[0];   // R: P(Pi)
     float* sa = P->vec[1];   // P0
     float* cc = P->vec[7];   // Z: diffusivity
-    k_vol_pi<<<vgrid(d1, h1, w1), VTHREADS, 0, s>>>(u1, d1, h1, w1, u2, P->ds[l - 2], P->hs[l - 2],
-                                                    P->ws[l - 2], ue);
-    k_vol_quad<<<vgrid(d, h, w), VTHREADS, 0, s>>>(ue, d1, h1, w1, ut, d, h, w);
+    VCK(launch_vol_pi(u1, d1, h1, w1, u2, P->ds[l - 2], P->hs[l - 2], P->ws[l - 2], ue, s));
+    VCK(launch_vol_quad(ue, d1, h1, w1, ut, d, h, w, s));
     const int steps = P->opt.diffusion_steps;
     float* cur = steps == 0 ? out : sa;
-    k_vol_smooth<<<vgrid(d, h, w), VTHREADS, 0, s>>>(ut, d, h, w, (float)P->opt.s_scale, cur);
+    VCK(launch_vol_smooth(ut, d, h, w, (float)P->opt.s_scale, cur, s));
     const float ik2 = (float)(1.0 / (P->kpm * P->kpm));
     for (int st = 0; st < steps; ++st) {
         float* nxt = st == steps - 1 ? out : (cur == sa ? ut : sa);
-        k_vol_pm_c<<<vgrid(d, h, w), VTHREADS, 0, s>>>(cur, d, h, w, ik2, cc);
-        k_vol_pm_step<<<vgrid(d, h, w), VTHREADS, 0, s>>>(cur, cc, d, h, w, (float)P->tau, nxt);
+        VCK(launch_vol_denoise(cur, d, h, w, ik2, (float)P->tau, cc, nxt, s));
         cur = nxt;
     }
-    VCK(cudaGetLastError());
     return EECMG_OK;
 }
 
@@ -688,13 +497,15 @@ eecmg_status eecmg_vol_plan(int width, int height, int depth, int levels, const 
     P->grid.resize(L);
     int maxgrid = 1;
     for (int l = 0; l < L; ++l) {
-        const int r = std::max(P->taps[l].r, P->tapsT[l].r);
-        const size_t smem = std::max(tile_bytes(P->taps[l]), tile_bytes(P->tapsT[l]));
+        // the attribute belongs to the kernel, which plans of every form share
+        const int r = P->taps[l].r;
+        const size_t most = std::max(form_bytes(r, VF_SEP), std::max(form_bytes(r, VF_DENSE), form_bytes(r, VF_SPARSE)));
+        const size_t smem = form_bytes(r, P->taps[l].form);
         e = cudaFuncSetAttribute(vol_kernels().solve[r], cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)smem);
+                                 (int)most);
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(vol_kernels().apply[r], cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)smem);
+                                     (int)most);
         int per = 0;
         if (e == cudaSuccess)
             e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, vol_kernels().solve[r], NTHREADS, smem);
@@ -702,11 +513,8 @@ eecmg_status eecmg_vol_plan(int width, int height, int depth, int levels, const 
             delete P;
             return set_error(EECMG_ERR_CUDA, "eecmg_vol_plan: level solve does not fit an SM");
         }
-        VolJob J{};
-        J.d = P->ds[l];
-        J.h = P->hs[l];
-        J.w = P->ws[l];
-        const long long want = std::max<long long>(level_tiles(J), (P->n4[l] + NTHREADS - 1) / NTHREADS);
+        const long long want =
+            std::max<long long>(level_units(P->ds[l], P->hs[l], P->ws[l], P->taps[l]), (P->n4[l] + NTHREADS - 1) / NTHREADS);
         const long long cap = (long long)per * P->sms;
         P->grid[l] = (int)std::max<long long>(1, std::min(want, cap));
         maxgrid = std::max(maxgrid, P->grid[l]);
@@ -857,9 +665,7 @@ eecmg_status eecmg_vol_smooth(eecmg_vol_t P, int level, const float* x, float* y
     eecmg_status st = check_level(P, level, "eecmg_vol_smooth");
     if (st != EECMG_OK) return st;
     if (!x || !y || x == y) return set_error(EECMG_ERR_INVALID_ARG, "eecmg_vol_smooth: bad buffers");
-    k_vol_smooth<<<vgrid(P->ds[level], P->hs[level], P->ws[level]), VTHREADS, 0, s>>>(x, P->ds[level], P->hs[level], P->ws[level],
-                                                        (float)P->opt.s_scale, y);
-    VCK(cudaGetLastError());
+    VCK(launch_vol_smooth(x, P->ds[level], P->hs[level], P->ws[level], (float)P->opt.s_scale, y, s));
     return EECMG_OK;
 }
 
@@ -868,10 +674,7 @@ eecmg_status eecmg_vol_denoise(eecmg_vol_t P, int level, const float* x, float* 
     if (st != EECMG_OK) return st;
     if (!x || !y || x == y) return set_error(EECMG_ERR_INVALID_ARG, "eecmg_vol_denoise: bad buffers");
     const int d = P->ds[level], h = P->hs[level], w = P->ws[level];
-    k_vol_pm_c<<<vgrid(d, h, w), VTHREADS, 0, s>>>(x, d, h, w, (float)(1.0 / (P->kpm * P->kpm)),
-                                                      P->vec[7]);
-    k_vol_pm_step<<<vgrid(d, h, w), VTHREADS, 0, s>>>(x, P->vec[7], d, h, w, (float)P->tau, y);
-    VCK(cudaGetLastError());
+    VCK(launch_vol_denoise(x, d, h, w, (float)(1.0 / (P->kpm * P->kpm)), (float)P->tau, P->vec[7], y, s));
     return EECMG_OK;
 }
 

@@ -16,15 +16,23 @@ namespace vol {
 
 constexpr int VR = EECMG_VOL_MAX_RADIUS;
 constexpr int VK = 2 * VR + 1;
-constexpr int TX = 32, TY = 8, TZ = 8;  // output tile (columns, rows, slices)
+constexpr int MX = 64;                  // columns of a marched tile
+constexpr int TX = 32, TY = 8, TZ = 8;  // sparse form: output tile (columns, rows, slices)
+
+// How a level's PSF is applied (fixed by the planner from its taps).
+enum VolForm : int {
+    VF_SEP = 0,     // an outer product of three factors: three 1-D passes
+    VF_DENSE = 1,   // rows of 2 r + 1 taps for every (slice, row) offset that has one
+    VF_SPARSE = 2,  // a list of taps
+};
 
 // Taps of one level in correlation form, y(v) = sum_d C(d) x(v + d), C(d) = K(-d),
 // centred at r = the level PSF's largest radius (shorter axes padded with zeros).
 struct VolTaps {
     int r;
-    int sep;                       // 1: C = cz (x) cy (x) cx
-    float cz[VK], cy[VK], cx[VK];  // factors, index d + r
-    int ntap;                      // general form: taps in the job's tap list
+    int form;                      // VolForm
+    float cz[VK], cy[VK], cx[VK];  // VF_SEP: factors, index d + r
+    int ntap;                      // else: taps in the job's tap list
 };
 
 struct VolJob {
@@ -38,7 +46,7 @@ struct VolJob {
     float* Q[3];
     float* Z;
     VolTaps taps;
-    const int4* gtaps;  // general form: (dz, dy, dx, weight bits)
+    const int4* gtaps;  // VF_DENSE, VF_SPARSE: (dz, dy, dx, weight bits)
     int m;
     int zero_start;
     double stop_tol;    // discrepancy: stop once ||r||_RMS <= stop_tol (0: off)
@@ -48,219 +56,14 @@ struct VolJob {
     double* out;        // [0] iterations, [1] ||r||^2, [2] stop reason
 };
 
-// Per-block replica of the solve's scalars (identical in every block).
+// Per-block replica of the solve's scalars (identical in every block), as
+// double-float pairs: on GB300 a dependent FP64 operation takes 66 cycles, and the
+// divisions and roots of these updates took 4-6 us of every phase in FP64.
 struct VolScal {
-    double rr, gg, qq, qqp, qqn, a, b1, b2;
+    DF rr, qq, qqp, qqn, lim2;
+    float a, b1, b2;
     int k, done;
 };
-
-// -------------------------------------------------------------------- tile
-//
-// A block loops over its output tiles t = blockIdx.x, + gridDim.x, ...  The
-// input window of a tile (the tile plus an r-voxel halo, zero outside the
-// volume) is fetched with cp.async (16-byte chunks where rows are 16-byte
-// aligned, else 4-byte copies; zero fill past the volume) into one of two
-// shared-memory buffers while the previous tile is convolved from the other.
-// The separable form runs three passes in shared memory: slices over every
-// staged (row, column) into B, rows over B into C (C reuses the tile's own
-// input buffer), columns over C; the first two slide a register window along
-// their axis, so each staged value is read once.  The general form sums its
-// tap list over the window.
-
-template <int R>
-struct VolTile {
-    // a staged row starts PADX = R rounded up to 4 voxels left of the tile, so
-    // rows are whole 16-byte chunks; voxel x of the window sits at X0 + x
-    static constexpr int PADX = (R + 3) / 4 * 4, X0 = PADX - R;
-    static constexpr int NZ = TZ + 2 * R, NY = TY + 2 * R, AX = TX + 2 * PADX;
-    static constexpr int IN = NZ * NY * AX;  // one input buffer
-    static constexpr int MID = TZ * NY * AX; // B: the slice pass's output
-    static constexpr size_t bytes(bool sep) { return sizeof(float) * (2 * (size_t)IN + (sep ? MID : 0)); }
-};
-
-__device__ __forceinline__ int num_tiles(const VolJob& J) {
-    return ((J.w + TX - 1) / TX) * ((J.h + TY - 1) / TY) * ((J.d + TZ - 1) / TZ);
-}
-
-__device__ __forceinline__ void tile_origin(const VolJob& J, int t, int& x0, int& y0, int& z0) {
-    const int ntx = (J.w + TX - 1) / TX, nty = (J.h + TY - 1) / TY;
-    x0 = (t % ntx) * TX;
-    y0 = ((t / ntx) % nty) * TY;
-    z0 = (t / ntx / nty) * TZ;
-}
-
-template <int R>
-__device__ __forceinline__ void stage_tile(const VolJob& J, const float* __restrict__ x, int t, float* A) {
-    using T = VolTile<R>;
-    int x0, y0, z0;
-    tile_origin(J, t, x0, y0, z0);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const unsigned int base = (unsigned int)__cvta_generic_to_shared(A);
-    if ((J.w & 3) == 0 && (reinterpret_cast<uintptr_t>(x) & 15) == 0) {
-        // 16-byte chunks: rows are 16-byte aligned in memory (w a multiple of 4,
-        // x 16-byte aligned) and a chunk is
-        // either inside the row or wholly past one of its ends (zero fill)
-        constexpr int CH = T::AX / 4;           // chunks per row
-        constexpr int RPW = 32 / CH;            // rows per warp instruction
-        constexpr int ROWS = T::NZ * T::NY;
-        const int sub = lane / CH, c = lane - sub * CH;
-        for (int r0 = warp * RPW; r0 < ROWS; r0 += (NTHREADS / 32) * RPW) {
-            const int row = r0 + sub;
-            if (sub >= RPW || row >= ROWS) continue;
-            const int za = row / T::NY, ya = row - za * T::NY;
-            const int gz = z0 - R + za, gy = y0 - R + ya, gx = x0 - T::PADX + 4 * c;
-            const bool in = gz >= 0 && gz < J.d && gy >= 0 && gy < J.h && gx >= 0 && gx < J.w;
-            const float* g = in ? x + ((long long)gz * J.h + gy) * J.w + gx : x;
-            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(
-                             base + 4u * (unsigned int)(row * T::AX + 4 * c)),
-                         "l"(g), "r"(in ? 16 : 0)
-                         : "memory");
-        }
-    } else {
-        for (int row = warp; row < T::NZ * T::NY; row += NTHREADS / 32) {
-            const int za = row / T::NY, ya = row - za * T::NY;
-            const int gz = z0 - R + za, gy = y0 - R + ya;
-            const bool rin = gz >= 0 && gz < J.d && gy >= 0 && gy < J.h;
-            const float* src = x + ((long long)(rin ? gz : 0) * J.h + (rin ? gy : 0)) * J.w;
-#pragma unroll
-            for (int xa = lane; xa < T::AX; xa += 32) {
-                const int gx = x0 - T::PADX + xa;
-                const bool in = rin && gx >= 0 && gx < J.w;
-                const float* g = in ? src + gx : x;  // a valid address either way
-                asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(
-                                 base + 4u * (unsigned int)(row * T::AX + xa)),
-                             "l"(g), "r"(in ? 4 : 0)
-                             : "memory");
-            }
-        }
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-}
-
-// Convolves the staged tile t (buffer A) and calls epi(voxel index, (H x)(v))
-// for every in-volume output.  Ends with __syncthreads().
-template <int R, class Epi>
-__device__ __forceinline__ void compute_tile(const VolJob& J, int t, float* A, float* B, Epi&& epi) {
-    using T = VolTile<R>;
-    const VolTaps& K = J.taps;
-    int x0, y0, z0;
-    tile_origin(J, t, x0, y0, z0);
-    const int xo = threadIdx.x & 31, warp = threadIdx.x >> 5;  // warp = output row within a slice
-    const int gx = x0 + xo, gy = y0 + warp;
-    // the epilogue's read-only operands of this thread's outputs, fetched
-    // before the passes so that their latency hides behind the convolution
-    const bool col_in = gy < J.h && gx < J.w;
-    float2 pre[TZ];
-#pragma unroll
-    for (int zo = 0; zo < TZ; ++zo)
-        pre[zo] = (col_in && z0 + zo < J.d) ? epi.pre(((long long)(z0 + zo) * J.h + gy) * J.w + gx)
-                                            : make_float2(0.f, 0.f);
-    if (K.sep) {
-        // slices first: B[z][y][x] = sum_dz cz A[z + dz][y][x] for the TZ output
-        // slices, every staged (y, x) column; each thread slides a register
-        // window down its column, so a staged value is read once
-        constexpr int COLS = T::NY * T::AX;
-        for (int c = threadIdx.x; c < COLS; c += NTHREADS) {
-            float win[T::NZ];
-#pragma unroll
-            for (int z = 0; z < T::NZ; ++z) win[z] = A[z * COLS + c];
-#pragma unroll
-            for (int zo = 0; zo < TZ; ++zo) {
-                float s = 0.f;
-#pragma unroll
-                for (int o = 0; o <= 2 * R; ++o) s = fmaf(K.cz[o], win[zo + o], s);
-                B[zo * COLS + c] = s;
-            }
-        }
-        __syncthreads();
-        // rows: C[z][y][x] = sum_dy cy B[z][y + dy][x] for the TY output rows,
-        // every (z, x) column (C over the window's own buffer)
-        float* C = A;
-        constexpr int COLS2 = TZ * T::AX;
-        for (int c = threadIdx.x; c < COLS2; c += NTHREADS) {
-            const int z = c / T::AX, x = c - z * T::AX;
-            const float* b = B + z * COLS + x;
-            float win[T::NY];
-#pragma unroll
-            for (int y = 0; y < T::NY; ++y) win[y] = b[y * T::AX];
-#pragma unroll
-            for (int yo = 0; yo < TY; ++yo) {
-                float s = 0.f;
-#pragma unroll
-                for (int p = 0; p <= 2 * R; ++p) s = fmaf(K.cy[p], win[yo + p], s);
-                C[(z * TY + yo) * T::AX + x] = s;
-            }
-        }
-        __syncthreads();
-        // columns: out[z][y][x] = sum_dx cx C[z][y][X0 + x + dx]
-        float s[TZ];
-#pragma unroll
-        for (int zo = 0; zo < TZ; ++zo) {
-            s[zo] = 0.f;
-            const float* c = C + (zo * TY + warp) * T::AX + T::X0 + xo;
-#pragma unroll
-            for (int q = 0; q <= 2 * R; ++q) s[zo] = fmaf(K.cx[q], c[q], s[zo]);
-        }
-        if (col_in) {
-#pragma unroll
-            for (int zo = 0; zo < TZ; ++zo)
-                if (z0 + zo < J.d) epi(((long long)(z0 + zo) * J.h + gy) * J.w + gx, s[zo], pre[zo]);
-        }
-    } else {
-#pragma unroll
-        for (int zo = 0; zo < TZ; ++zo) {
-            const float* a = A + ((zo + R) * T::NY + warp + R) * T::AX + T::X0 + xo + R;
-            float s = 0.f;
-            for (int k = 0; k < K.ntap; ++k) {
-                const int4 tp = __ldg(J.gtaps + k);
-                s = fmaf(__int_as_float(tp.w), a[(tp.x * T::NY + tp.y) * T::AX + tp.z], s);
-            }
-            if (z0 + zo < J.d && col_in) epi(((long long)(z0 + zo) * J.h + gy) * J.w + gx, s, pre[zo]);
-        }
-    }
-    __syncthreads();  // the buffers are restaged after this
-}
-
-// An epilogue: pre(v) loads the operands output v needs (at most two floats,
-// issued before the convolution), op(v, (H x)(v), operands) consumes them.
-template <class Pre, class Op>
-struct Epilogue {
-    Pre pre;
-    Op op;
-    __device__ __forceinline__ void operator()(long long v, float hx, float2 p) { op(v, hx, p); }
-};
-template <class Pre, class Op>
-__device__ __forceinline__ Epilogue<Pre, Op> epilogue(Pre pre, Op op) {
-    return Epilogue<Pre, Op>{pre, op};
-}
-__device__ __forceinline__ float2 no_pre(long long) { return make_float2(0.f, 0.f); }
-
-// One convolution phase: H x over all the block's tiles, the next tile's
-// window in flight while the current one is convolved.
-template <int R, class Epi>
-__device__ __forceinline__ void conv_phase(const VolJob& J, const float* __restrict__ x, float* sm,
-                                           Epi&& epi) {
-    using T = VolTile<R>;
-    const int ntiles = num_tiles(J), nb = gridDim.x;
-    int t = blockIdx.x;
-    if (t >= ntiles) return;  // the whole block
-    float* B = sm + 2 * T::IN;
-    int buf = 0;
-    stage_tile<R>(J, x, t, sm);
-    for (; t < ntiles; t += nb) {
-        if (t + nb < ntiles) {
-            stage_tile<R>(J, x, t + nb, sm + (buf ^ 1) * T::IN);
-            asm volatile("cp.async.wait_group 1;" ::: "memory");
-        } else {
-            asm volatile("cp.async.wait_group 0;" ::: "memory");
-        }
-        __syncthreads();
-        compute_tile<R>(J, t, sm + buf * T::IN, B, epi);
-        buf ^= 1;
-    }
-}
-
-
 
 // per-thread compensated sum (cascaded: the rounding errors are kept in lo)
 __device__ __forceinline__ void acc_add(DF& a, float v) {
@@ -269,8 +72,467 @@ __device__ __forceinline__ void acc_add(DF& a, float v) {
     a.lo += s.lo;
 }
 
-__device__ __forceinline__ double tot2(const DF (&t)[4], int j) {
-    return df_to_double(t[2 * j]) + df_to_double(t[2 * j + 1]);
+// ------------------------------------------------------------- convolution
+//
+// A convolution phase divides the level's slices of MX x MY column tiles evenly
+// over the blocks: block b takes a contiguous range of the (tile, slice) pairs,
+// and within a tile marches along the slices.  A ring of input planes (the tile
+// with an r-voxel halo, zero outside the volume) is filled by cp.async three
+// slices ahead; one barrier per slice.
+// VF_SEP: a thread owns four columns of one or two rows, halo columns included.
+// The rows pass reads the staged plane; its result enters the 2 r + 1 outputs along
+// the slices it contributes to, kept as partial sums in registers; a finished
+// slice goes through shared memory once for the columns pass, one slice behind.
+// So a voxel costs 3 (2 r + 1) multiplications, about a quarter of a shared
+// load per multiplication and no index arithmetic beyond its row.
+// VF_DENSE: the thread's window of each row enters all 2 r + 1 slices' partial sums.
+// A range repeats the 2 r slices around its start, 2 r / 54 of the work at 256^3.
+// What a phase does with H x: out = H x (or a - H x) and its sums.
+enum VolEpi : int { VE_RESID = 0, VE_STORE, VE_Q1, VE_Z };
+struct EpiArgs {
+    const float* a;  // VE_RESID: g; VE_Q1: r; VE_Z: q_k
+    const float* b;  // VE_Z: q_{k-1} (NULL: none)
+    float* out;
+    int mode;
+};
+
+__device__ __forceinline__ float4 ld_quad(const float* p, size_t i, int nv, bool vec) {
+    if (vec) return __ldcg(reinterpret_cast<const float4*>(p + i));
+    float4 r = make_float4(0.f, 0.f, 0.f, 0.f);
+    r.x = __ldcg(p + i);
+    if (nv > 1) r.y = __ldcg(p + i + 1);
+    if (nv > 2) r.z = __ldcg(p + i + 2);
+    if (nv > 3) r.w = __ldcg(p + i + 3);
+    return r;
+}
+
+// Four outputs of a row at element i, of which nv (1..4) lie in the volume; their
+// products are added to sa, sb.
+__device__ __forceinline__ void epilogue4(const EpiArgs& E, size_t i, int nv, bool vec, float4 hx, float4 a,
+                                          float4 b, float& sa, float& sb) {
+    if (nv < 4) hx.w = a.w = 0.f;
+    if (nv < 3) hx.z = a.z = 0.f;
+    if (nv < 2) hx.y = a.y = 0.f;
+    float4 o = hx;
+    if (E.mode == VE_RESID) {
+        o = make_float4(a.x - hx.x, a.y - hx.y, a.z - hx.z, a.w - hx.w);
+        sa = dot4(o, o, sa);
+        sb = dot4(a, a, sb);
+    } else if (E.mode == VE_Q1) {
+        sa = dot4(hx, hx, sa);
+        sb = dot4(a, hx, sb);
+    } else if (E.mode == VE_Z) {
+        sa = dot4(a, hx, sa);
+        sb = dot4(b, hx, sb);
+    }
+    if (vec) {
+        *reinterpret_cast<float4*>(E.out + i) = o;
+    } else {
+        E.out[i] = o.x;
+        if (nv > 1) E.out[i + 1] = o.y;
+        if (nv > 2) E.out[i + 2] = o.z;
+        if (nv > 3) E.out[i + 3] = o.w;
+    }
+}
+
+template <int R>
+struct March {
+    // a staged row starts PADX = R rounded up to 4 voxels left of the tile, so
+    // rows are whole 16-byte chunks
+    static constexpr int PADX = (R + 3) / 4 * 4;
+    static constexpr int AX = MX + 2 * PADX, QX = AX / 4;  // a staged row, in floats and in quads
+    static constexpr int RING = 4;
+    // VF_SEP: RPT rows per thread (two quads of 2 r partial sums fit the registers up to
+    // r = 4), QX quads x GR row groups of threads
+    static constexpr int RPT = R <= 4 ? 2 : 1, GR = NTHREADS / QX, SY = GR * RPT;
+    static constexpr int SPLANE = (SY + 2 * R) * AX, V = SY * AX;
+    // VF_DENSE: 16 quads x 16 rows of threads
+    static constexpr int DY = NTHREADS / (MX / 4), DPLANE = (DY + 2 * R) * AX;
+    static constexpr int NW4 = (2 * R + 1 + 3) / 4;        // a row of taps, padded to float4
+    static constexpr int WTS = (2 * R + 1) * (2 * R + 1) * NW4 * 4;
+    static constexpr size_t bytes(int form) {
+        return sizeof(float) * (form == VF_SEP ? RING * (size_t)SPLANE + 2 * V : RING * (size_t)DPLANE + WTS + 16);
+    }
+    static constexpr int rows(int form) { return form == VF_SEP ? SY : DY; }
+};
+
+// The copies of one window plane (NY x AX floats) that a thread issues: offsets
+// within a slice and validity are the same for every slice of a segment.
+template <int NY, int AX>
+struct PlaneCopies {
+    static constexpr int N16 = (NY * AX / 4 + NTHREADS - 1) / NTHREADS;
+    int off[N16];        // 16-byte chunks: element offset in the slice; < 0: outside (zero)
+    int y0, x0;          // the window's first row and column
+    __device__ __forceinline__ void set(const VolJob& J, int y, int x) {
+        y0 = y;
+        x0 = x;
+#pragma unroll
+        for (int k = 0; k < N16; ++k) {
+            const int c = threadIdx.x + k * NTHREADS, r = c / (AX / 4), gy = y + r, gx = x + 4 * (c - r * (AX / 4));
+            const bool in = c < NY * AX / 4 && gy >= 0 && gy < J.h && gx >= 0 && gx < J.w;
+            off[k] = in ? gy * J.w + gx : -1;  // a slice has fewer than 2^31 elements
+        }
+    }
+    __device__ __forceinline__ void issue(const VolJob& J, const float* __restrict__ x, int z, float* A, bool vec) const {
+        const unsigned int base = smem_u32(A);
+        const bool zin = z >= 0 && z < J.d;
+        const float* src = x + (long long)(zin ? z : 0) * J.h * J.w;
+        if (vec) {
+#pragma unroll
+            for (int k = 0; k < N16; ++k) {
+                const int c = threadIdx.x + k * NTHREADS;
+                const bool in = zin && off[k] >= 0;
+                if (c < NY * AX / 4)
+                    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(base + 16u * (unsigned int)c),
+                                 "l"(in ? src + off[k] : x), "r"(in ? 16 : 0)
+                                 : "memory");
+            }
+        } else {
+            // a warp per row (rows start anywhere)
+            const int lane = threadIdx.x & 31;
+            for (int r = threadIdx.x >> 5; r < NY; r += NTHREADS / 32) {
+                const int gy = y0 + r;
+                const bool rin = zin && gy >= 0 && gy < J.h;
+                const float* row = src + (long long)(rin ? gy : 0) * J.w;
+#pragma unroll
+                for (int c = lane; c < AX; c += 32) {
+                    const int gx = x0 + c;
+                    const bool in = rin && gx >= 0 && gx < J.w;
+                    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(
+                                     base + 4u * (unsigned int)(r * AX + c)),
+                                 "l"(in ? row + gx : x), "r"(in ? 4 : 0)
+                                 : "memory");
+                }
+            }
+        }
+    }
+};
+
+__device__ __forceinline__ void commit_copies() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void wait_copies() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+__device__ __forceinline__ float elem(const float4& v, int k) {
+    return k == 0 ? v.x : (k == 1 ? v.y : (k == 2 ? v.z : v.w));
+}
+__device__ __forceinline__ bool aligned16(const void* a, const void* b, const void* c) {
+    return ((reinterpret_cast<uintptr_t>(a) | reinterpret_cast<uintptr_t>(b) | reinterpret_cast<uintptr_t>(c)) & 15) == 0;
+}
+
+// One segment of a phase's range: slices z0 .. z1 - 1 of the tile at (y0, x0).
+struct Segment {
+    int y0, x0, z0, z1;
+};
+template <int SY>
+__device__ __forceinline__ bool next_segment(const VolJob& J, long long& u, long long u_end, Segment& g) {
+    if (u >= u_end) return false;
+    const int ntx = (J.w + MX - 1) / MX, tile = (int)(u / J.d);
+    g.z0 = (int)(u - (long long)tile * J.d);
+    g.z1 = (int)min((long long)J.d, g.z0 + (u_end - u));
+    g.x0 = (tile % ntx) * MX;
+    g.y0 = (tile / ntx) * SY;
+    u += g.z1 - g.z0;
+    return true;
+}
+__device__ __forceinline__ long long tile_units(const VolJob& J, int sy) {
+    return (long long)((J.w + MX - 1) / MX) * ((J.h + sy - 1) / sy) * J.d;
+}
+
+// One convolution phase of a separable PSF, out = epilogue(C (*) x).
+template <int R>
+__device__ __forceinline__ void sep_phase(const VolJob& J, const float* __restrict__ x, float* sm, const EpiArgs& E,
+                                          DF (&acc)[2]) {
+    using M = March<R>;
+    constexpr int RPT = M::RPT, QX = M::QX, HQ = M::PADX / 4;
+    const int tid = threadIdx.x, q = tid % QX, g = tid / QX;  // quad of the staged row, row group
+    const bool work = g < M::GR, main = work && q >= HQ && q < QX - HQ;
+    float* V = sm + M::RING * M::SPLANE;
+    const long long units = tile_units(J, M::SY);
+    long long u = units * blockIdx.x / gridDim.x;
+    const long long u_end = units * (blockIdx.x + 1) / gridDim.x;
+    const bool vin = (J.w & 3) == 0 && aligned16(x, nullptr, nullptr);
+    const bool vec = (J.w & 3) == 0 && aligned16(E.a, E.b, E.out);
+    const size_t sl = (size_t)J.h * J.w;
+    PlaneCopies<M::SY + 2 * R, M::AX> P;
+    Segment G;
+    while (next_segment<M::SY>(J, u, u_end, G)) {
+        const int gx = G.x0 + 4 * (q - HQ), gy = G.y0 + g * RPT;
+        int nv[RPT];  // outputs of each row inside the volume (<= 0: none)
+#pragma unroll
+        for (int i = 0; i < RPT; ++i) nv[i] = main && gy + i < J.h ? min(4, J.w - gx) : 0;
+        const int s0 = G.z0 - R, s_end = G.z1 + R;  // input slices
+        P.set(J, G.y0 - R, G.x0 - M::PADX);
+        __syncthreads();  // the ring and V of the segment before
+#pragma unroll
+        for (int k = 0; k < M::RING; ++k) {
+            if (s0 + k < s_end) P.issue(J, x, s0 + k, sm + k * M::SPLANE, vin);
+            commit_copies();
+        }
+        constexpr int NP = R > 0 ? 2 * R : 1;
+        float4 part[RPT][NP];  // partial sums of the outputs s - R + k before slice s
+#pragma unroll
+        for (int i = 0; i < RPT; ++i)
+#pragma unroll
+            for (int k = 0; k < NP; ++k) part[i][k] = make_float4(0.f, 0.f, 0.f, 0.f);
+        float4 own[RPT];  // the finished slice's quads, waiting for the columns pass
+        int slot = 0;
+        size_t at = ((size_t)G.z0 * J.h + gy) * J.w + gx;
+#pragma unroll 1
+        for (int s = s0; s <= s_end; ++s, slot = (slot + 1) & (M::RING - 1)) {
+            // the slice finished one step ago: z = s - 1 - R
+            const bool emit = s - 1 - R >= G.z0;
+            float4 pa[RPT], pb[RPT];
+#pragma unroll
+            for (int i = 0; i < RPT; ++i) {
+                pa[i] = pb[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (emit && nv[i] > 0) {
+                    if (E.a) pa[i] = ld_quad(E.a, at + (size_t)(i * J.w), nv[i], vec);
+                    if (E.b) pb[i] = ld_quad(E.b, at + (size_t)(i * J.w), nv[i], vec);
+                }
+            }
+            wait_copies<M::RING - 2>();  // plane s (and s + 1) has landed
+            __syncthreads();             // V of slice s - 1 is complete; the slot of plane s - 1 is free
+            if (s > s0) {
+                if (s + M::RING - 1 < s_end)
+                    P.issue(J, x, s + M::RING - 1, sm + ((slot + M::RING - 1) & (M::RING - 1)) * M::SPLANE, vin);
+                commit_copies();
+            }
+            const int b = slot & 1;
+            if (emit && main) {  // columns pass
+                const float4* v = reinterpret_cast<const float4*>(V + (b ^ 1) * M::V) + g * RPT * QX + q;
+                float sa = 0.f, sb = 0.f;
+#pragma unroll
+                for (int i = 0; i < RPT; ++i) {
+                    float w[4 * (2 * HQ + 1)];
+#pragma unroll
+                    for (int j = 0; j <= 2 * HQ; ++j) {
+                        const float4 t = j == HQ ? own[i] : v[i * QX + j - HQ];
+                        w[4 * j] = t.x;
+                        w[4 * j + 1] = t.y;
+                        w[4 * j + 2] = t.z;
+                        w[4 * j + 3] = t.w;
+                    }
+                    float o[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                    for (int k = 0; k <= 2 * R; ++k)
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) o[c] = fmaf(J.taps.cx[k], w[M::PADX - R + c + k], o[c]);
+                    if (nv[i] > 0)
+                        epilogue4(E, at + (size_t)(i * J.w), nv[i], vec, make_float4(o[0], o[1], o[2], o[3]),
+                                  pa[i], pb[i], sa, sb);
+                }
+                acc_add(acc[0], sa);
+                acc_add(acc[1], sb);
+            }
+            if (emit) at += sl;
+            if (s < s_end && work) {  // rows pass, then along the slices
+                const float4* a = reinterpret_cast<const float4*>(sm + slot * M::SPLANE) + g * RPT * QX + q;
+                float4 h[RPT];
+#pragma unroll
+                for (int i = 0; i < RPT; ++i) h[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+                for (int p = 0; p < 2 * R + RPT; ++p) {
+                    const float4 t = a[p * QX];
+#pragma unroll
+                    for (int i = 0; i < RPT; ++i)
+                        if (p - i >= 0 && p - i <= 2 * R) h[i] = fma4(J.taps.cy[p - i], t, h[i]);
+                }
+                float4* v = reinterpret_cast<float4*>(V + b * M::V) + g * RPT * QX + q;
+#pragma unroll
+                for (int i = 0; i < RPT; ++i) {
+                    if constexpr (R == 0) {
+                        own[i] = mul4(J.taps.cz[0], h[i]);
+                    } else {
+                        own[i] = fma4(J.taps.cz[2 * R], h[i], part[i][0]);
+#pragma unroll
+                        for (int k = 0; k < 2 * R - 1; ++k) part[i][k] = fma4(J.taps.cz[2 * R - 1 - k], h[i], part[i][k + 1]);
+                        part[i][2 * R - 1] = mul4(J.taps.cz[0], h[i]);
+                    }
+                    v[i * QX] = own[i];
+                }
+            }
+        }
+    }
+    wait_copies<0>();
+}
+
+// One convolution phase of a PSF with dense rows of taps.
+template <int R>
+__device__ __forceinline__ void dense_phase(const VolJob& J, const float* __restrict__ x, float* sm, const EpiArgs& E,
+                                            DF (&acc)[2]) {
+    using M = March<R>;
+    const int tid = threadIdx.x, q = tid & 15, row = tid >> 4;  // four columns of one row
+    float* W = sm + M::RING * M::DPLANE;                        // W[((dy + R) (2R + 1) + dz + R) 4 NW4 + dx + R]
+    unsigned int* mask = reinterpret_cast<unsigned int*>(W + M::WTS);  // slice offsets with taps, by row offset
+    const long long units = tile_units(J, M::DY);
+    long long u = units * blockIdx.x / gridDim.x;
+    const long long u_end = units * (blockIdx.x + 1) / gridDim.x;
+    const bool vin = (J.w & 3) == 0 && aligned16(x, nullptr, nullptr);
+    const bool vec = (J.w & 3) == 0 && aligned16(E.a, E.b, E.out);
+    for (int i = tid; i < M::WTS; i += NTHREADS) W[i] = 0.f;
+    if (tid < 16) mask[tid] = 0u;
+    __syncthreads();
+    for (int k = tid; k < J.taps.ntap; k += NTHREADS) {
+        const int4 t = __ldg(J.gtaps + k);
+        W[((t.y + R) * (2 * R + 1) + t.x + R) * (4 * M::NW4) + t.z + R] = __int_as_float(t.w);
+        atomicOr(&mask[t.y + R], 1u << (t.x + R));
+    }
+    PlaneCopies<M::DY + 2 * R, M::AX> P;
+    Segment G;
+    while (next_segment<M::DY>(J, u, u_end, G)) {
+        const int gx = G.x0 + 4 * q, gy = G.y0 + row;
+        const int nv = gy < J.h ? min(4, J.w - gx) : 0;  // outputs inside the volume (<= 0: none)
+        const int s0 = max(G.z0 - R, 0), s_end = min(G.z1 + R, J.d);  // input slices (those outside are zero)
+        P.set(J, G.y0 - R, G.x0 - M::PADX);
+        __syncthreads();  // the taps; the ring of the segment before
+#pragma unroll
+        for (int k = 0; k < M::RING; ++k) {
+            if (s0 + k < s_end) P.issue(J, x, s0 + k, sm + k * M::DPLANE, vin);
+            commit_copies();
+        }
+        float4 part[2 * R + 1];  // partial sums of the outputs z = s - R + k
+#pragma unroll
+        for (int k = 0; k <= 2 * R; ++k) part[k] = make_float4(0.f, 0.f, 0.f, 0.f);
+        int slot = 0;
+#pragma unroll 1
+        for (int s = s0; s < G.z1 + R; ++s, slot = (slot + 1) & (M::RING - 1)) {
+            // the epilogue's operands of output slice s - R, fetched ahead
+            const int z = s - R;
+            const bool emit = z >= G.z0 && nv > 0;
+            const size_t at = ((size_t)(z >= G.z0 ? z : G.z0) * J.h + gy) * J.w + gx;
+            float4 pa = make_float4(0.f, 0.f, 0.f, 0.f), pb = pa;
+            if (emit && E.a) pa = ld_quad(E.a, at, nv, vec);
+            if (emit && E.b) pb = ld_quad(E.b, at, nv, vec);
+            wait_copies<M::RING - 2>();  // plane s has landed
+            __syncthreads();             // the slot of plane s - 1 is free
+            if (s > s0) {
+                if (s + M::RING - 1 < s_end)
+                    P.issue(J, x, s + M::RING - 1, sm + ((slot + M::RING - 1) & (M::RING - 1)) * M::DPLANE, vin);
+                commit_copies();
+            }
+            // slice offsets whose output lies in the segment: k = z - s + R for z in [z0, z1)
+            const int k_lo = max(G.z0 - z, 0), k_hi = min(G.z1 - 1 - z, 2 * R);
+            const unsigned int seg = s < s_end && k_lo <= k_hi ? ((2u << (2 * R - k_lo)) - 1u) & ~((1u << (2 * R - k_hi)) - 1u) : 0u;
+            constexpr int NQ = (4 + 2 * M::PADX) / 4;
+            const float* A = sm + slot * M::DPLANE;
+#pragma unroll 1
+            for (int p = 0; p <= 2 * R; ++p) {
+                const unsigned int mk = mask[p] & seg;
+                if (mk == 0u) continue;
+                const float4* a = reinterpret_cast<const float4*>(A + (row + p) * M::AX) + q;
+                float w[4 * NQ];
+#pragma unroll
+                for (int j = 0; j < NQ; ++j) {
+                    const float4 v = a[j];
+                    w[4 * j] = v.x;
+                    w[4 * j + 1] = v.y;
+                    w[4 * j + 2] = v.z;
+                    w[4 * j + 3] = v.w;
+                }
+                const float4* Wp = reinterpret_cast<const float4*>(W) + p * (2 * R + 1) * M::NW4;
+#pragma unroll
+                for (int k = 0; k <= 2 * R; ++k) {  // slice offset R - k: output z = s - R + k
+                    if ((mk >> (2 * R - k)) & 1u) {
+#pragma unroll
+                        for (int j = 0; j < M::NW4; ++j) {
+                            const float4 t = Wp[(2 * R - k) * M::NW4 + j];
+#pragma unroll
+                            for (int e = 0; e < 4; ++e)
+                                if (4 * j + e <= 2 * R) {
+                                    constexpr int o = M::PADX - R;
+                                    part[k].x = fmaf(elem(t, e), w[o + 4 * j + e], part[k].x);
+                                    part[k].y = fmaf(elem(t, e), w[o + 1 + 4 * j + e], part[k].y);
+                                    part[k].z = fmaf(elem(t, e), w[o + 2 + 4 * j + e], part[k].z);
+                                    part[k].w = fmaf(elem(t, e), w[o + 3 + 4 * j + e], part[k].w);
+                                }
+                        }
+                    }
+                }
+            }
+            if (emit) {
+                float sa = 0.f, sb = 0.f;
+                epilogue4(E, at, nv, vec, part[0], pa, pb, sa, sb);
+                acc_add(acc[0], sa);
+                acc_add(acc[1], sb);
+            }
+#pragma unroll
+            for (int k = 0; k < 2 * R; ++k) part[k] = part[k + 1];
+            part[2 * R] = make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+    }
+    wait_copies<0>();
+}
+
+// VF_SPARSE: few taps in a large support.  8 x 8 x 32 output tiles, staged with
+// their halo; every output sums the tap list over the window.
+template <int R>
+struct SparseTile {
+    static constexpr int NZ = TZ + 2 * R, NY = TY + 2 * R, AX = TX + 2 * R;
+    static constexpr size_t bytes = sizeof(float) * (size_t)NZ * NY * AX;
+};
+template <int R>
+__device__ __forceinline__ void sparse_phase(const VolJob& J, const float* __restrict__ x, float* A, const EpiArgs& E,
+                                             DF (&acc)[2]) {
+    using S = SparseTile<R>;
+    const int ntx = (J.w + TX - 1) / TX, nty = (J.h + TY - 1) / TY;
+    const int ntiles = ntx * nty * ((J.d + TZ - 1) / TZ);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned int base = smem_u32(A);
+    for (int t = blockIdx.x; t < ntiles; t += gridDim.x) {
+        const int x0 = (t % ntx) * TX, y0 = ((t / ntx) % nty) * TY, z0 = (t / ntx / nty) * TZ;
+        __syncthreads();
+        for (int r = warp; r < S::NZ * S::NY; r += NTHREADS / 32) {
+            const int gz = z0 - R + r / S::NY, gy = y0 - R + r % S::NY;
+            const bool rin = gz >= 0 && gz < J.d && gy >= 0 && gy < J.h;
+            const float* src = x + ((long long)(rin ? gz : 0) * J.h + (rin ? gy : 0)) * J.w;
+            for (int c = lane; c < S::AX; c += 32) {
+                const int gx = x0 - R + c;
+                const bool in = rin && gx >= 0 && gx < J.w;
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(
+                                 base + 4u * (unsigned int)(r * S::AX + c)),
+                             "l"(in ? src + gx : x), "r"(in ? 4 : 0)
+                             : "memory");
+            }
+        }
+        asm volatile("cp.async.commit_group;\n\tcp.async.wait_group 0;" ::: "memory");
+        __syncthreads();
+        const int gx = x0 + lane, gy = y0 + warp;
+        float s[TZ];
+#pragma unroll
+        for (int z = 0; z < TZ; ++z) s[z] = 0.f;
+        const float* a = A + (R * S::NY + warp + R) * S::AX + lane + R;
+        for (int k = 0; k < J.taps.ntap; ++k) {
+            const int4 tp = __ldg(J.gtaps + k);
+            const float* b = a + (tp.x * S::NY + tp.y) * S::AX + tp.z;
+#pragma unroll
+            for (int z = 0; z < TZ; ++z) s[z] = fmaf(__int_as_float(tp.w), b[z * S::NY * S::AX], s[z]);
+        }
+        if (gx < J.w && gy < J.h) {
+#pragma unroll
+            for (int z = 0; z < TZ; ++z) {
+                if (z0 + z >= J.d) break;
+                const size_t i = ((size_t)(z0 + z) * J.h + gy) * J.w + gx;
+                const float4 va = make_float4(E.a ? __ldcg(E.a + i) : 0.f, 0.f, 0.f, 0.f);
+                const float4 vb = make_float4(E.b ? __ldcg(E.b + i) : 0.f, 0.f, 0.f, 0.f);
+                float sa = 0.f, sb = 0.f;
+                epilogue4(E, i, 1, false, make_float4(s[z], 0.f, 0.f, 0.f), va, vb, sa, sb);
+                acc_add(acc[0], sa);
+                acc_add(acc[1], sb);
+            }
+        }
+    }
+}
+
+template <int R>
+__device__ __forceinline__ void conv_phase(const VolJob& J, const float* __restrict__ x, float* sm, const EpiArgs& E,
+                                           DF (&acc)[2]) {
+    if (J.taps.form == VF_SEP)
+        sep_phase<R>(J, x, sm, E, acc);
+    else if (J.taps.form == VF_DENSE)
+        dense_phase<R>(J, x, sm, E, acc);
+    else
+        sparse_phase<R>(J, x, sm, E, acc);
 }
 
 // A vector phase over float4 elements i = gtid, gtid + gstr, ...: two elements
@@ -304,14 +566,7 @@ __device__ __forceinline__ void vec_phase(long long n4, long long gtid, long lon
 
 // ------------------------------------------------------------- level solve
 
-// Stop test of the oracle's level smoother, checked before every iteration.
-__device__ __forceinline__ bool level_done(const VolJob& J, double rr, double gg) {
-    if (J.stop_tol > 0.0 && sqrt(rr / (double)J.n) <= J.stop_tol) return true;
-    if (J.conv_tol > 0.0 && sqrt(rr) <= J.conv_tol * sqrt(gg)) return true;
-    return false;
-}
-
-__device__ __forceinline__ bool pos_finite(double x) { return x > 0.0 && isfinite(x); }
+__device__ __forceinline__ bool df_pos_finite(DF x) { return x.hi > 0.f && df_finite(x); }
 
 // MR-II (the three-term recurrence of the oracle's level smoother):
 //   r0 = g - H u0;  p1 = H r0, q1 = H p1, a = <r,q>/<q,q>, u += a p, r -= a q;
@@ -319,24 +574,19 @@ __device__ __forceinline__ bool pos_finite(double x) { return x > 0.0 && isfinit
 //   z = H q_k, b1 = <z,q_k>/<q_k,q_k>, b2 = <z,q_{k-1}>/<q_{k-1},q_{k-1}> (k >= 2),
 //   q_{k+1} = z - b1 q_k - b2 q_{k-1}, p_{k+1} = q_k - b1 p_k - b2 p_{k-1},
 //   a = <r,q_{k+1}>/<q_{k+1},q_{k+1}>, u += a p_{k+1}, r -= a q_{k+1}.
-// p and q live in rings of three buffers: p_k = P[(k - 1) % 3].
+// p and q live in rings of three buffers: p_k = P[(k - 1) % 3].  The phases run in
+// one loop with one convolution, one update and one reduction in the code: on the
+// small levels a phase's first execution is bound by the fetch of its instructions.
+enum VolPhase : int { PH_ZERO = 0, PH_R0, PH_P1, PH_Q1, PH_Z, PH_DIR, PH_UPD };
+
 template <int R>
-__global__ void __launch_bounds__(NTHREADS, 2) k_vol_mr2(VolJob J) {
+__global__ void __launch_bounds__(NTHREADS, 2) k_vol_mr2(const __grid_constant__ VolJob J) {
     extern __shared__ __align__(16) float sm[];
     __shared__ VolScal S;
     const unsigned int nb = gridDim.x, bid = blockIdx.x;
     const long long gtid = (long long)bid * NTHREADS + threadIdx.x, gstr = (long long)nb * NTHREADS;
-    unsigned int phase = 0;
-    bool ok = true;
-    auto reduce = [&](const DF (&acc)[2], auto&& fin) {
-        float v[4] = {acc[0].hi, acc[0].lo, acc[1].hi, acc[1].lo};
-        return grid_reduce<4>(v, J.partials, J.gs, nb, bid, phase++, fin);
-    };
     float4* u4 = reinterpret_cast<float4*>(J.u);
     float4* r4 = reinterpret_cast<float4*>(J.R);
-    const float4* g4 = reinterpret_cast<const float4*>(J.g);
-
-    // r0 = g - H u0 (a zero start writes u = 0, r = g); ||r||^2, ||g||^2
     {
         // the vector phases run on whole float4s: zero the (at most 3) padding
         // voxels past n of every vector this solve reads, whatever an earlier
@@ -353,106 +603,20 @@ __global__ void __launch_bounds__(NTHREADS, 2) k_vol_mr2(VolJob J) {
                 J.Q[b][i] = 0.f;
             }
         }
+    }
+    unsigned int phase = 0;
+    bool ok = true;
+    int kind = J.zero_start ? PH_ZERO : PH_R0;
+#pragma unroll 1
+    for (;;) {
         DF acc[2] = {{0.f, 0.f}, {0.f, 0.f}};
-        if (J.zero_start) {
-            for (long long i = gtid; i < J.n4; i += gstr) {
-                const float4 g = __ldcg(g4 + i);
-                u4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-                r4[i] = g;
-                acc_add(acc[0], dot4(g, g, 0.f));
-                acc_add(acc[1], dot4(g, g, 0.f));
-            }
-        } else {
-            conv_phase<R>(J, J.u, sm, epilogue(
-                [&](long long i) { return make_float2(__ldcg(J.g + i), 0.f); },
-                [&](long long i, float hx, float2 p) {
-                    const float g = p.x;
-                    const float r = g - hx;
-                    J.R[i] = r;
-                    acc_add(acc[0], r * r);
-                    acc_add(acc[1], g * g);
-                }));
-        }
-        ok = reduce(acc, [&](const DF (&t)[4]) {
-            S.rr = tot2(t, 0);
-            S.gg = tot2(t, 1);
-            S.k = 0;
-            S.done = (J.m <= 0 || level_done(J, S.rr, S.gg)) ? 1 : 0;
-        });
-    }
-    if (ok && !S.done) {
-        // p1 = H r0
-        conv_phase<R>(J, J.R, sm, epilogue(no_pre, [&](long long i, float hx, float2) { J.P[0][i] = hx; }));
-        DF none[2] = {{0.f, 0.f}, {0.f, 0.f}};
-        ok = reduce(none, [&](const DF (&)[4]) {});
-    }
-    if (ok && !S.done) {
-        // q1 = H p1; <q,q>, <r,q>
-        DF acc[2] = {{0.f, 0.f}, {0.f, 0.f}};
-        conv_phase<R>(J, J.P[0], sm, epilogue(
-            [&](long long i) { return make_float2(__ldcg(J.R + i), 0.f); },
-            [&](long long i, float hx, float2 p) {
-                J.Q[0][i] = hx;
-                acc_add(acc[0], hx * hx);
-                acc_add(acc[1], p.x * hx);
-            }));
-        ok = reduce(acc, [&](const DF (&t)[4]) {
-            const double qq = tot2(t, 0), rq = tot2(t, 1);
-            if (!pos_finite(qq)) {
-                S.done = 2;
-            } else {
-                S.qq = qq;
-                S.a = rq / qq;
-            }
-        });
-    }
-    if (ok && !S.done) {
-        // u += a p1, r -= a q1; ||r||^2
-        DF acc[2] = {{0.f, 0.f}, {0.f, 0.f}};
-        const float a = (float)S.a;
-        const float4* const in[4] = {reinterpret_cast<const float4*>(J.P[0]),
-                                     reinterpret_cast<const float4*>(J.Q[0]), u4, r4};
-        float4* const out[2] = {u4, r4};
-        vec_phase<4, 2>(J.n4, gtid, gstr, in, out, [&](const float4 (&x)[4], float4 (&y)[2]) {
-            y[0] = fma4(a, x[0], x[2]);
-            y[1] = fma4(-a, x[1], x[3]);
-            acc_add(acc[0], dot4(y[1], y[1], 0.f));
-        });
-        ok = reduce(acc, [&](const DF (&t)[4]) {
-            S.rr = tot2(t, 0);
-            S.k = 1;
-            S.qqp = 0.0;
-            S.done = (S.k >= J.m || level_done(J, S.rr, S.gg)) ? 1 : 0;
-        });
-    }
-    while (ok && !S.done) {
-        const int k = S.k;
-        const int cur = (k - 1) % 3, prv = (k + 1) % 3, nxt = k % 3;
-        const float* q = J.Q[cur];
-        const float* qp = J.Q[prv];
-        const bool two = k >= 2;
-        // z = H q_k; <z, q_k>, <z, q_{k-1}>
-        {
-            DF acc[2] = {{0.f, 0.f}, {0.f, 0.f}};
-            conv_phase<R>(J, q, sm, epilogue(
-                [&](long long i) { return make_float2(__ldcg(q + i), two ? __ldcg(qp + i) : 0.f); },
-                [&](long long i, float hx, float2 p) {
-                    J.Z[i] = hx;
-                    acc_add(acc[0], hx * p.x);
-                    if (two) acc_add(acc[1], hx * p.y);
-                }));
-            ok = reduce(acc, [&](const DF (&t)[4]) {
-                S.b1 = tot2(t, 0) / S.qq;
-                S.b2 = two ? tot2(t, 1) / S.qqp : 0.0;
-            });
-            if (!ok) break;
-        }
-        // q_{k+1}, p_{k+1}; <q_{k+1}, q_{k+1}>, <r, q_{k+1}>
-        {
-            DF acc[2] = {{0.f, 0.f}, {0.f, 0.f}};
-            const float b1 = (float)S.b1, b2 = (float)S.b2;
+        const int k = kind >= PH_Z ? S.k : 0;  // PH_Z, PH_DIR: from q_k to q_{k+1}; PH_UPD: applies step k + 1
+        const int cur = (k + 2) % 3, prv = (k + 1) % 3, nxt = k % 3;  // buffers of steps k, k - 1, k + 1
+        if (kind == PH_DIR) {
+            // q_{k+1}, p_{k+1}; <q_{k+1}, q_{k+1}>, <r, q_{k+1}>
+            const float b1 = S.b1, b2 = S.b2;
             float4* const out[2] = {reinterpret_cast<float4*>(J.Q[nxt]), reinterpret_cast<float4*>(J.P[nxt])};
-            if (two) {
+            if (k >= 2) {
                 const float4* const in[6] = {reinterpret_cast<const float4*>(J.Z),
                                              reinterpret_cast<const float4*>(J.Q[cur]),
                                              reinterpret_cast<const float4*>(J.P[cur]), r4,
@@ -475,21 +639,9 @@ __global__ void __launch_bounds__(NTHREADS, 2) k_vol_mr2(VolJob J) {
                     acc_add(acc[1], dot4(x[3], y[0], 0.f));
                 });
             }
-            ok = reduce(acc, [&](const DF (&t)[4]) {
-                const double qqn = tot2(t, 0), rqn = tot2(t, 1);
-                if (!pos_finite(qqn)) {
-                    S.done = 2;
-                } else {
-                    S.qqn = qqn;
-                    S.a = rqn / qqn;
-                }
-            });
-            if (!ok || S.done) break;
-        }
-        // u += a p_{k+1}, r -= a q_{k+1}; ||r||^2
-        {
-            DF acc[2] = {{0.f, 0.f}, {0.f, 0.f}};
-            const float a = (float)S.a;
+        } else if (kind == PH_UPD) {
+            // u += a p_{k+1}, r -= a q_{k+1}; ||r||^2
+            const float a = S.a;
             const float4* const in[4] = {reinterpret_cast<const float4*>(J.P[nxt]),
                                          reinterpret_cast<const float4*>(J.Q[nxt]), u4, r4};
             float4* const out[2] = {u4, r4};
@@ -498,36 +650,90 @@ __global__ void __launch_bounds__(NTHREADS, 2) k_vol_mr2(VolJob J) {
                 y[1] = fma4(-a, x[1], x[3]);
                 acc_add(acc[0], dot4(y[1], y[1], 0.f));
             });
-            ok = reduce(acc, [&](const DF (&t)[4]) {
-                S.rr = tot2(t, 0);
+        } else if (kind == PH_ZERO) {
+            // a zero start: u = 0, r = g
+            const float4* g4 = reinterpret_cast<const float4*>(J.g);
+            for (long long i = gtid; i < J.n4; i += gstr) {
+                const float4 g = __ldcg(g4 + i);
+                u4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+                r4[i] = g;
+                acc_add(acc[0], dot4(g, g, 0.f));
+            }
+            acc[1] = acc[0];
+        } else {
+            // r0 = g - H u0 | p1 = H r0 | q1 = H p1 | z = H q_k, with the sums each needs
+            const float* x = kind == PH_R0 ? J.u : (kind == PH_P1 ? J.R : (kind == PH_Q1 ? J.P[0] : J.Q[cur]));
+            EpiArgs E;
+            E.mode = kind - PH_R0 + VE_RESID;
+            E.a = kind == PH_R0 ? J.g : (kind == PH_P1 ? nullptr : (kind == PH_Q1 ? J.R : J.Q[cur]));
+            E.b = kind == PH_Z && k >= 2 ? J.Q[prv] : nullptr;
+            E.out = kind == PH_R0 ? J.R : (kind == PH_P1 ? J.P[0] : (kind == PH_Q1 ? J.Q[0] : J.Z));
+            conv_phase<R>(J, x, sm, E, acc);
+        }
+        ok = grid_reduce_df<2>(acc, J.partials, J.gs, nb, bid, phase++, [&](const DF (&t)[2]) {
+            if (kind <= PH_R0) {
+                S.rr = t[0];
+                S.k = 0;
+                // the limit of both rules, formed once (off the later phases' path)
+                const double gg = df_to_double(t[1]);
+                const double l1 = J.conv_tol * J.conv_tol * gg, l2 = J.stop_tol * J.stop_tol * (double)J.n;
+                S.lim2 = df_from_double(l1 > l2 ? l1 : l2);
+                const bool rule = J.stop_tol > 0.0 || J.conv_tol > 0.0;
+                if (!rule) S.lim2 = DF{-1.f, 0.f};
+                S.done = (J.m <= 0 || df_le(S.rr, S.lim2)) ? 1 : 0;
+            } else if (kind == PH_Q1) {
+                S.done = df_pos_finite(t[0]) ? 0 : 2;
+                S.qqn = t[0];
+                S.a = df_div(t[1], t[0]).hi;
+            } else if (kind == PH_Z) {
+                S.b1 = df_div(t[0], S.qq).hi;
+                S.b2 = k >= 2 ? df_div(t[1], S.qqp).hi : 0.f;
+            } else if (kind == PH_DIR) {
+                S.done = df_pos_finite(t[0]) ? 0 : 2;
+                S.qqn = t[0];
+                S.a = df_div(t[1], t[0]).hi;
+            } else if (kind == PH_UPD) {
+                S.rr = t[0];
                 S.qqp = S.qq;
                 S.qq = S.qqn;
-                S.k = S.k + 1;
-                S.done = (S.k >= J.m || level_done(J, S.rr, S.gg)) ? 1 : 0;
-            });
-        }
+                S.k = k + 1;
+                S.done = (S.k >= J.m || df_le(S.rr, S.lim2)) ? 1 : 0;
+            }
+        });
+        if (!ok || S.done) break;
+        kind = kind == PH_ZERO || kind == PH_R0 ? PH_P1
+               : kind == PH_P1                  ? PH_Q1
+               : kind == PH_Q1 || kind == PH_DIR ? PH_UPD
+               : kind == PH_UPD                 ? PH_Z
+                                                : PH_DIR;
     }
     if (bid == 0 && threadIdx.x == 0) {
         J.out[0] = S.k;
-        J.out[1] = S.rr;
+        J.out[1] = df_to_double(S.rr);
         J.out[2] = ok ? S.done : -1;
     }
     grid_exit(J.gs, nb);
 }
 
-// H x (or H^T x with the transposed taps) of a whole level, one tile per block.
+// H x (or H^T x with the transposed taps) of a whole level.
 template <int R>
-__global__ void __launch_bounds__(NTHREADS) k_vol_apply(VolJob J, const float* __restrict__ x,
-                                                        float* __restrict__ y) {
+__global__ void __launch_bounds__(NTHREADS, 2) k_vol_apply(const __grid_constant__ VolJob J,
+                                                           const float* __restrict__ x, float* __restrict__ y) {
     extern __shared__ __align__(16) float sm[];
-    stage_tile<R>(J, x, blockIdx.x, sm);
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-    __syncthreads();
-    compute_tile<R>(J, blockIdx.x, sm, sm + 2 * VolTile<R>::IN,
-                    epilogue(no_pre, [&](long long i, float hx, float2) { y[i] = hx; }));
+    DF acc[2] = {{0.f, 0.f}, {0.f, 0.f}};
+    conv_phase<R>(J, x, sm, EpiArgs{nullptr, nullptr, y, VE_STORE}, acc);
 }
 
-// ------------------------------------------------------------ level start
+// Shared memory of the solve and apply kernels of radius r, and the rows of the
+// tiles whose slices a phase divides over the blocks.
+template <int R>
+constexpr size_t vol_smem(int form) {
+    return form == VF_SPARSE ? SparseTile<R>::bytes : March<R>::bytes(form);
+}
+template <int R>
+constexpr int vol_tile_rows(int form) {
+    return March<R>::rows(form);
+}
 
 // The solve and apply kernels of radius r (0 .. EECMG_VOL_MAX_RADIUS), from the
 // translation unit that instantiates them; false if r is outside its range.
