@@ -91,25 +91,79 @@ eecmg_status plan_waves(const std::vector<std::pair<eecmg_plan_s*, int>>& items,
         cur.bf16 = bf;
         cur.cluster = cl;
         cur.resident = res;
+        // cooperative jobs: the largest first, each into the first wave with room (a
+        // wave takes the time of its slowest job however full it is)
+        std::vector<std::pair<int, int>> order;  // (blocks, item)
         for (int i : kv.second) {
             const LevelPlan& Lp = items[i].first->lv[items[i].second];
-            const int nb = cl > 0 ? cl : std::max(1, std::min(cap, level_shape(Lp.h, Lp.w, Lp.rt, cg, bf).blocks));
-            if ((long long)cur.blocks + nb > cap && !cur.jobs.empty()) {  // next wave
-                waves.push_back(cur);
-                cur.jobs.clear();
-                cur.block_job.clear();
-                cur.blocks = 0;
-            }
-            LevelJob J = make_job(items[i].first, items[i].second);
-            J.block0 = cur.blocks;
-            J.nblocks = nb;
-            for (int b = 0; b < nb; ++b) cur.block_job.push_back((unsigned short)cur.jobs.size());
-            cur.jobs.push_back(J);
-            cur.blocks += nb;
+            order.push_back({cl > 0 ? cl : std::max(1, std::min(cap, level_shape(Lp.h, Lp.w, Lp.rt, cg, bf).blocks)), i});
         }
-        if (!cur.jobs.empty()) waves.push_back(cur);
+        if (cl == 0)
+            std::stable_sort(order.begin(), order.end(),
+                             [](const std::pair<int, int>& x, const std::pair<int, int>& y) { return x.first > y.first; });
+        const size_t first = waves.size();
+        for (const auto& o : order) {
+            size_t w = first;
+            while (w < waves.size() && (long long)waves[w].blocks + o.first > cap) ++w;
+            if (w == waves.size()) waves.push_back(cur);
+            HostWave& W = waves[w];
+            LevelJob J = make_job(items[o.second].first, items[o.second].second);
+            J.block0 = W.blocks;
+            J.nblocks = o.first;
+            for (int b = 0; b < o.first; ++b) W.block_job.push_back((unsigned short)W.jobs.size());
+            W.jobs.push_back(J);
+            W.blocks += o.first;
+        }
     }
     return EECMG_OK;
+}
+
+cudaError_t Fan::create() {
+    cudaError_t e = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);
+    for (int i = 0; i < SIDES && e == cudaSuccess; ++i) {
+        e = cudaStreamCreateWithFlags(&side[i], cudaStreamNonBlocking);
+        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&join[i], cudaEventDisableTiming);
+    }
+    return e;
+}
+
+void Fan::destroy() {
+    for (int i = 0; i < SIDES; ++i) {
+        if (side[i]) cudaStreamDestroy(side[i]);
+        if (join[i]) cudaEventDestroy(join[i]);
+        side[i] = nullptr;
+        join[i] = nullptr;
+    }
+    if (fork) cudaEventDestroy(fork);
+    fork = nullptr;
+}
+
+void Fan::begin(cudaStream_t s) {
+    main_ = s;
+    n_ = 0;
+    forked_ = false;
+}
+
+cudaError_t Fan::next(cudaStream_t* out) {
+    cudaError_t e = cudaSuccess;
+    if (!forked_) e = cudaEventRecord(fork, main_);
+    forked_ = true;
+    const int i = n_ % SIDES;
+    if (e == cudaSuccess && n_ < SIDES) e = cudaStreamWaitEvent(side[i], fork, 0);
+    ++n_;
+    *out = side[i];
+    return e;
+}
+
+cudaError_t Fan::end() {
+    cudaError_t e = cudaSuccess;
+    for (int i = 0; i < SIDES && i < n_; ++i) {
+        cudaError_t r = cudaEventRecord(join[i], side[i]);
+        if (r == cudaSuccess) r = cudaStreamWaitEvent(main_, join[i], 0);
+        if (e == cudaSuccess) e = r;
+    }
+    n_ = 0;
+    return e;
 }
 
 void add_op(std::vector<OpGroup>& groups, size_t gi, int op, OpItem it) {
@@ -274,12 +328,11 @@ struct BatchCtx {
     cudaStream_t cap_stream = nullptr;
     cudaGraphExec_t gexec = nullptr;
     size_t graph_nodes = 0;  // kernel nodes of one batched restoration
-    // Steps 0 and 1 (the two levels solved from zero, Algorithm 2) run as two
-    // branches of the graph when every job of both is a resident solve: such
+    // Steps 0 and 1 (the two levels solved from zero, Algorithm 2) run side by
+    // side when every job of both is a resident solve: such
     // a solve touches only its own level's g, u, scalars and sync words.
     bool fork01 = false;
-    cudaStream_t side = nullptr;
-    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+    Fan fan;
     // Measurement hook: event-record nodes around the level-solve launches of
     // cascade step timed_step (-1: none).
     int timed_step = -1;
@@ -303,9 +356,7 @@ struct BatchCtx {
     ~BatchCtx() {
         if (gexec) cudaGraphExecDestroy(gexec);
         if (cap_stream) cudaStreamDestroy(cap_stream);
-        if (side) cudaStreamDestroy(side);
-        if (ev_fork) cudaEventDestroy(ev_fork);
-        if (ev_join) cudaEventDestroy(ev_join);
+        fan.destroy();
         for (cudaEvent_t e : tev)
             if (e) cudaEventDestroy(e);
         if (dmem) cudaFree(dmem);
@@ -450,11 +501,7 @@ eecmg_status build_ctx(BatchCtx& C) {
             ok = level_shape(P->lv[l].h, P->lv[l].w, P->lv[l].rt, cg, bf).resident > 0;
         C.fork01 = C.fork01 && ok;
     }
-    if (C.fork01 &&
-        (cudaStreamCreateWithFlags(&C.side, cudaStreamNonBlocking) != cudaSuccess ||
-         cudaEventCreateWithFlags(&C.ev_fork, cudaEventDisableTiming) != cudaSuccess ||
-         cudaEventCreateWithFlags(&C.ev_join, cudaEventDisableTiming) != cudaSuccess))
-        return set_error(EECMG_ERR_CUDA, "eecmg_restore_batched: side stream");
+    if (C.fan.create() != cudaSuccess) return set_error(EECMG_ERR_CUDA, "eecmg_restore_batched: side streams");
     return EECMG_OK;
 }
 
@@ -466,13 +513,35 @@ eecmg_status build_ctx(BatchCtx& C) {
                                                  ": " + cudaGetErrorString(e_));               \
     } while (0)
 
-eecmg_status enqueue_step(BatchCtx& C, int st, cudaStream_t s) {
-    for (const OpLaunch& L : C.step_ops[st]) BCK(launch_ops_batch(L.op, L.d_items, L.n, L.blocks, s));
+// The level solves of steps st .. st + n - 1 (independent of each other), cluster
+// waves on the side streams; the side streams always join back into s.
+eecmg_status enqueue_waves(BatchCtx& C, int st, int n, cudaStream_t s) {
+    C.fan.begin(s);
+    cudaError_t e = cudaSuccess;
+    // clusters first: they are short, and a cooperative wave may need every SM
+    for (int pass = 0; pass < 2; ++pass)
+        for (int k = st; k < st + n; ++k)
+            for (auto& w : C.steps[k]) {
+                if (e != cudaSuccess || (w.cluster > 0) != (pass == 0)) continue;
+                cudaStream_t t = s;
+                if (w.cluster > 0) e = C.fan.next(&t);
+                if (e == cudaSuccess)
+                    e = launch_level_batch(w.d_jobs, w.d_block_job, w.njobs, w.blocks, w.rt, w.sep, w.prec, w.cgls,
+                                           w.bf16, w.cluster, w.resident, t);
+            }
+    const cudaError_t j = C.fan.end();
+    BCK(e);
+    BCK(j);
+    return EECMG_OK;
+}
+
+eecmg_status enqueue_step(BatchCtx& C, int st, int n, cudaStream_t s) {
+    for (int k = st; k < st + n; ++k)
+        for (const OpLaunch& L : C.step_ops[k]) BCK(launch_ops_batch(L.op, L.d_items, L.n, L.blocks, s));
     const bool timed = st == C.timed_step && !C.steps[st].empty();
     if (timed) BCK(cudaEventRecordWithFlags(C.tev[0], s, cudaEventRecordExternal));
-    for (auto& w : C.steps[st])
-        BCK(launch_level_batch(w.d_jobs, w.d_block_job, w.njobs, w.blocks, w.rt, w.sep, w.prec, w.cgls,
-                               w.bf16, w.cluster, w.resident, s));
+    eecmg_status e = enqueue_waves(C, st, n, s);
+    if (e != EECMG_OK) return e;
     if (timed) BCK(cudaEventRecordWithFlags(C.tev[1], s, cudaEventRecordExternal));
     return EECMG_OK;
 }
@@ -480,18 +549,13 @@ eecmg_status enqueue_step(BatchCtx& C, int st, cudaStream_t s) {
 eecmg_status enqueue_batch(BatchCtx& C, cudaStream_t s) {
     for (const OpLaunch& L : C.restrict_ops) BCK(launch_ops_batch(L.op, L.d_items, L.n, L.blocks, s));
     int st = 0;
-    if (C.fork01) {  // step 0 on the side branch, step 1 on the main one
-        BCK(cudaEventRecord(C.ev_fork, s));
-        BCK(cudaStreamWaitEvent(C.side, C.ev_fork, 0));
-        eecmg_status e0 = enqueue_step(C, 0, C.side);
-        eecmg_status e1 = e0 == EECMG_OK ? enqueue_step(C, 1, s) : e0;
-        BCK(cudaEventRecord(C.ev_join, C.side));  // always join the branch back
-        BCK(cudaStreamWaitEvent(s, C.ev_join, 0));
-        if (e1 != EECMG_OK) return e1;
+    if (C.fork01 && C.timed_step != 0 && C.timed_step != 1) {
+        eecmg_status e = enqueue_step(C, 0, 2, s);
+        if (e != EECMG_OK) return e;
         st = 2;
     }
     for (; st < (int)C.steps.size(); ++st) {
-        eecmg_status e = enqueue_step(C, st, s);
+        eecmg_status e = enqueue_step(C, st, 1, s);
         if (e != EECMG_OK) return e;
     }
     return EECMG_OK;

@@ -157,6 +157,7 @@ struct eecmg_server_s {
     char* arena_mem = nullptr;
     Arena arena;
     cudaStream_t stream = nullptr;
+    Fan fan;  // side streams of the cluster waves
     // job tables of the ticks in flight
     size_t ring_bytes = 0;
     char* d_ring = nullptr;  // RING x ring_bytes, device
@@ -374,12 +375,24 @@ eecmg_status enqueue_tick(eecmg_server_s* S, const std::vector<Request*>& admitt
         for (const Placed& p : rops_l[r])
             SCK(launch_ops_batch(p.op, (const OpItem*)(d + p.at), p.n, p.blocks, s));
         const auto& waves = rwaves[r];
-        for (size_t w = 0; w < waves.size(); ++w) {
-            const HostWave& W = waves[w];
-            SCK(launch_level_batch((const LevelJob*)(d + jo[r][w]), (const unsigned short*)(d + bo[r][w]),
-                                   (int)W.jobs.size(), W.blocks, W.rt, W.sep, W.prec, W.cgls, W.bf16,
-                                   W.cluster, W.resident, s));
-        }
+        // the cluster waves beside each other and beside the cooperative chain (a lone wave
+        // stays on the server's stream)
+        S->fan.begin(s);
+        cudaError_t we = cudaSuccess;
+        for (int pass = 0; pass < 2; ++pass)
+            for (size_t w = 0; w < waves.size(); ++w) {
+                const HostWave& W = waves[w];
+                if (we != cudaSuccess || (W.cluster > 0) != (pass == 0)) continue;
+                cudaStream_t t = s;
+                if (W.cluster > 0 && waves.size() > 1) we = S->fan.next(&t);
+                if (we == cudaSuccess)
+                    we = launch_level_batch((const LevelJob*)(d + jo[r][w]), (const unsigned short*)(d + bo[r][w]),
+                                            (int)W.jobs.size(), W.blocks, W.rt, W.sep, W.prec, W.cgls, W.bf16,
+                                            W.cluster, W.resident, t);
+            }
+        const cudaError_t je = S->fan.end();
+        SCK(we);
+        SCK(je);
         bool any = false;
         for (const Placed& p : rpost_l[r])
             SCK(launch_ops_batch(p.op, (const OpItem*)(d + p.at), p.n, p.blocks, s));
@@ -560,6 +573,7 @@ void free_server(eecmg_server_s* S) {
             if (S->rev[k][r]) cudaEventDestroy(S->rev[k][r]);
     if (S->base_ev) cudaEventDestroy(S->base_ev);
     if (S->stream) cudaStreamDestroy(S->stream);
+    S->fan.destroy();
     if (S->d_ring) cudaFree(S->d_ring);
     if (S->h_ring) cudaFreeHost(S->h_ring);
     if (S->h_stat) cudaFreeHost(S->h_stat);
@@ -599,6 +613,7 @@ eecmg_status eecmg_server_create(size_t mem_budget_bytes, int max_slots, eecmg_s
     S->ring_bytes = round256(tick_table_bound(max_slots, S->nsm));
     S->stat_stride = round256((sizeof(Scalars) + sizeof(GroupSync)) * MAX_LEVELS);
     e = cudaStreamCreateWithFlags(&S->stream, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = S->fan.create();
     if (e == cudaSuccess) e = cudaMalloc((void**)&S->d_ring, RING * S->ring_bytes);
     if (e == cudaSuccess) e = cudaMallocHost((void**)&S->h_ring, RING * S->ring_bytes);
     if (e == cudaSuccess) e = cudaMallocHost((void**)&S->h_stat, S->stat_stride * max_slots);
