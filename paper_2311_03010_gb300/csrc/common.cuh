@@ -18,6 +18,7 @@ namespace eecmg {
 constexpr int RMAX = EECMG_MAX_RADIUS;
 constexpr int KMAX = 2 * RMAX + 1;
 constexpr int TAPS_MAX = KMAX * KMAX;
+constexpr int RUN_MAX = 4;
 
 // One level's PSF in correlation form.  Device resident (plan-owned).
 struct Taps {
@@ -28,10 +29,34 @@ struct Taps {
     int pad[3];
     float cy[KMAX];       // separable factors, indexed by d + rt
     float cx[KMAX];
-    int dy[TAPS_MAX];     // non-zero taps (dy, dx, weight)
-    int dx[TAPS_MAX];
+    // the non-zero taps, by columns (dx ascending, dy ascending within): run[t] is the
+    // number of taps (1..RUN_MAX) of the vertical run that starts at t, 0 inside a run
+    short dy[TAPS_MAX], dx[TAPS_MAX], run[TAPS_MAX];
     float wt[TAPS_MAX];
 };
+
+// Fills the tap list of a correlation C(dy, dx), |dy| <= ry, |dx| <= rx, on the host.
+template <class F>
+inline void fill_taps(Taps* t, int ry, int rx, F&& C) {
+    int n = 0;
+    for (int dx = -rx; dx <= rx; ++dx)
+        for (int dy = -ry; dy <= ry; ++dy) {
+            const double v = C(dy, dx);
+            if (v == 0.0) continue;
+            t->dy[n] = (short)dy;
+            t->dx[n] = (short)dx;
+            t->wt[n] = (float)v;
+            t->run[n] = 0;
+            ++n;
+        }
+    t->ntap = n;
+    for (int a = 0; a < n;) {
+        int b = a + 1;
+        while (b < n && b - a < RUN_MAX && t->dx[b] == t->dx[a] && t->dy[b] == t->dy[b - 1] + 1) ++b;
+        t->run[a] = (short)(b - a);
+        a = b;
+    }
+}
 
 // A double-float value hi + lo (two floats, |lo| <= ulp(hi) / 2).
 struct DF {

@@ -5,7 +5,8 @@
 // The input tile plus a halo of R pixels is staged in shared memory (zero
 // outside the image: the block-Toeplitz boundary of Eq. 7).  Separable PSFs
 // run a vertical then a horizontal pass, each thread sliding a register
-// window over its outputs; other PSFs run over their non-zero taps.  PREC
+// window over its outputs; other PSFs run over their non-zero taps, a vertical run at
+// a time.  PREC
 // selects a compensated horizontal pass: each product is split exactly into
 // p + pe with an FMA, the p are summed with Kahan compensation and the pe in
 // a separate accumulator (7 FP32 operations per tap instead of 1).  The result
@@ -72,8 +73,9 @@ __device__ __forceinline__ void conv_stage_taps(ConvSmem<R, SEP>& S, const Taps*
         const int nt = taps->ntap;
         if (tid == 0) S.ntap = nt;
         for (int t = tid; t < nt; t += NTHREADS) {
-            // offset of tap (dy, dx) from window pixel (r, c) to (r + dy + R, c + dx + R)
-            S.off[t] = (taps->dy[t] + R) * ConvSmem<R, SEP>::IP + (taps->dx[t] + R);
+            // offset of tap (dy, dx) from window pixel (r, c) to (r + dy + R, c + dx + R), and
+            // the length of the run that starts there
+            S.off[t] = ((taps->dy[t] + R) * ConvSmem<R, SEP>::IP + (taps->dx[t] + R)) | (int)taps->run[t] << 16;
             S.wt[t] = taps->wt[t];
         }
     }
@@ -203,6 +205,47 @@ __device__ __forceinline__ void conv_load(ConvSmem<R, SEP>& S, const TIN* __rest
     conv_put<R, SEP, TIN>(S, V);
 }
 
+// A vertical run of N taps on NS staged tiles: N + 7 values of a column serve the 8
+// rows of each of the N taps from registers (one shared load per multiplication
+// was the bound of a tap at a time).  p[s]: tile s at the run's first tap for the
+// thread's first row; wt: the run's weights.  Motion blur, 15 pixels at 30 degrees:
+// 13 loads for 20 multiplications instead of 25.
+template <int N, int IP, int NS>
+__device__ __forceinline__ void conv_run(const float* const (&p)[NS], const float* wt, float (&acc)[NS][8]) {
+    float c[N];
+#pragma unroll
+    for (int j = 0; j < N; ++j) c[j] = wt[j];
+#pragma unroll
+    for (int s = 0; s < NS; ++s) {
+        float v[8 + N - 1];
+#pragma unroll
+        for (int i = 0; i < 8 + N - 1; ++i) v[i] = p[s][i * IP];
+#pragma unroll
+        for (int j = 0; j < N; ++j)
+#pragma unroll
+            for (int i = 0; i < 8; ++i) acc[s][i] = fmaf(c[j], v[i + j], acc[s][i]);
+    }
+}
+// Every run of the tap list (off, wt: S.off, S.wt): base[s] is tile s at the thread's
+// first row and column.
+template <int IP, int NS>
+__device__ __forceinline__ void conv_runs(const int* off, const float* wt, int nt, const float* const (&base)[NS],
+                                          float (&acc)[NS][8]) {
+    static_assert(RUN_MAX == 4, "one case per run length");
+#pragma unroll 1
+    for (int t = 0; t < nt;) {
+        const int o = off[t], n = o >> 16;
+        const float* p[NS];
+#pragma unroll
+        for (int s = 0; s < NS; ++s) p[s] = base[s] + (o & 0xffff);
+        if (n == 4) conv_run<4, IP, NS>(p, wt + t, acc);
+        else if (n == 3) conv_run<3, IP, NS>(p, wt + t, acc);
+        else if (n == 2) conv_run<2, IP, NS>(p, wt + t, acc);
+        else conv_run<1, IP, NS>(p, wt + t, acc);
+        t += n;
+    }
+}
+
 // Computes S.out from S.in (the caller synchronises before and after).
 template <int R, bool SEP, bool PREC>
 __device__ __forceinline__ void conv_compute(ConvSmem<R, SEP>& S) {
@@ -288,19 +331,13 @@ __device__ __forceinline__ void conv_compute(ConvSmem<R, SEP>& S) {
             S.out[r * PO + cg * 8 + i] = PREC ? __fadd_rn(acc[i], __fsub_rn(lo[i], comp[i])) : acc[i];
     } else {
         const int c = tid & 63, rg = tid >> 6;
-        float acc[8];
+        float acc[1][8];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) acc[i] = 0.f;
-        const int nt = S.ntap;
-        const float* base = S.in + SM::at(rg * 8, c);
-        for (int t = 0; t < nt; ++t) {
-            const float wt = S.wt[t];
-            const float* p = base + S.off[t];
+        for (int i = 0; i < 8; ++i) acc[0][i] = 0.f;
+        const float* const base[1] = {S.in + SM::at(rg * 8, c)};
+        conv_runs<SM::IP, 1>(S.off, S.wt, S.ntap, base, acc);
 #pragma unroll
-            for (int i = 0; i < 8; ++i) acc[i] = fmaf(wt, p[i * SM::IP], acc[i]);
-        }
-#pragma unroll
-        for (int i = 0; i < 8; ++i) S.out[(rg * 8 + i) * PO + c] = acc[i];
+        for (int i = 0; i < 8; ++i) S.out[(rg * 8 + i) * PO + c] = acc[0][i];
     }
 }
 

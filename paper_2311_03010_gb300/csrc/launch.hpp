@@ -103,6 +103,20 @@ int op_blocks_x(int op, int w);       // of which along x (OP_PSD: strips of col
 void place_starts(OpItem* items, int n);  // OP_PSD: sets th of the items of one launch
 cudaError_t launch_ops_batch(int op, const OpItem* d_items, int n, int total_blocks, cudaStream_t s);
 
+// Every coarse level of a data pyramid from the finest in one launch: level l's
+// pixel (a, b) is fine(step a, step b).
+struct RestrictLevels {
+    static constexpr int MAX = 29;  // levels below the finest
+    const float* fine = nullptr;
+    int wf = 0, n = 0;
+    struct {
+        float* out;
+        int h, w, step, block0, bx;
+    } lv[MAX];
+};
+// Appends a level (h x w, step) to R.
+void add_restrict(RestrictLevels& R, float* out, int h, int w, int step);
+cudaError_t launch_restrict_levels(const RestrictLevels& R, cudaStream_t s);
 cudaError_t launch_restrict(const float* fine, int hf, int wf, float* coarse, int hc, int wc,
                             cudaStream_t s);
 cudaError_t launch_extrapolate(const float* u1, int h1, int w1, const float* u2, int h2, int w2,

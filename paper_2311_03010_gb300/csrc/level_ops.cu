@@ -29,6 +29,17 @@ __global__ void k_restrict(const float* __restrict__ fine, int wf, float* __rest
     px_restrict(fine, wf, coarse, hc, wc, blockIdx.y * BY + threadIdx.y, blockIdx.x * BX + threadIdx.x);
 }
 
+// All coarse levels in one launch (a level alone is 3 us, nearly all of it launch): block
+// b serves the level whose block range holds it.
+__global__ void __launch_bounds__(BX* BY) k_restrict_levels(RestrictLevels R) {
+    const int blk = (int)blockIdx.x;
+    int l = 0;
+    while (l + 1 < R.n && R.lv[l + 1].block0 <= blk) ++l;
+    const int local = blk - R.lv[l].block0, by = local / R.lv[l].bx, bx = local - by * R.lv[l].bx;
+    px_restrict(R.fine, R.wf, R.lv[l].out, R.lv[l].h, R.lv[l].w, by * BY + threadIdx.y, bx * BX + threadIdx.x,
+                R.lv[l].step);
+}
+
 __device__ __forceinline__ void px_extrapolate(const float* __restrict__ u1, int h1, int w1,
                                                const float* __restrict__ u2, int h2, int w2,
                                                float* __restrict__ out, int a, int b) {
@@ -255,6 +266,26 @@ cudaError_t launch_restrict(const float* fine, int hf, int wf, float* coarse, in
     (void)hf;
     if (hc <= 0 || wc <= 0) return cudaSuccess;
     k_restrict<<<grid2(hc, wc), dim3(BX, BY), 0, s>>>(fine, wf, coarse, hc, wc);
+    return cudaGetLastError();
+}
+
+void add_restrict(RestrictLevels& R, float* out, int h, int w, int step) {
+    auto& v = R.lv[R.n];
+    v.out = out;
+    v.h = h;
+    v.w = w;
+    v.step = step;
+    const dim3 g = grid2(h, w);
+    v.bx = (int)g.x;
+    const auto* prev = R.n > 0 ? &R.lv[R.n - 1] : nullptr;
+    v.block0 = prev ? prev->block0 + op_blocks(OP_RESTRICT, prev->h, prev->w) : 0;
+    ++R.n;
+}
+
+cudaError_t launch_restrict_levels(const RestrictLevels& R, cudaStream_t s) {
+    if (R.n <= 0) return cudaSuccess;
+    const auto& last = R.lv[R.n - 1];
+    k_restrict_levels<<<last.block0 + op_blocks(OP_RESTRICT, last.h, last.w), dim3(BX, BY), 0, s>>>(R);
     return cudaGetLastError();
 }
 

@@ -210,15 +210,8 @@ __device__ __forceinline__ void conv_compute2(ConvSmem<R, SEP>& A, ConvSmem<R, S
         for (int s = 0; s < 2; ++s)
 #pragma unroll
             for (int i = 0; i < 8; ++i) acc[s][i] = 0.f;
-        const int nt = A.ntap;
-        for (int t = 0; t < nt; ++t) {
-            const float wt = A.wt[t];
-            const int off = A.off[t] + ConvSmem<R, SEP>::at(rg * 8, c);
-#pragma unroll
-            for (int s = 0; s < 2; ++s)
-#pragma unroll
-                for (int i = 0; i < 8; ++i) acc[s][i] = fmaf(wt, S[s]->in[off + i * ConvSmem<R, SEP>::IP], acc[s][i]);
-        }
+        const float* const base[2] = {A.in + SM::at(rg * 8, c), B.in + SM::at(rg * 8, c)};
+        conv_runs<SM::IP, 2>(A.off, A.wt, A.ntap, base, acc);
 #pragma unroll
         for (int s = 0; s < 2; ++s)
 #pragma unroll

@@ -111,18 +111,7 @@ extern "C" eecmg_status eecmg_residual_noalloc(int width, int height, const doub
     t.rx = rx;
     t.rt = ry > rx ? ry : rx;
     t.sep = 0;
-    int n = 0;
-    for (int dy = -ry; dy <= ry; ++dy)
-        for (int dx = -rx; dx <= rx; ++dx) {
-            const double v = psf[(size_t)(-dy + ry) * psf_w + (-dx + rx)];
-            if (v != 0.0) {
-                t.dy[n] = dy;
-                t.dx[n] = dx;
-                t.wt[n] = (float)v;
-                ++n;
-            }
-        }
-    t.ntap = n;
+    fill_taps(&t, ry, rx, [&](int dy, int dx) { return psf[(size_t)(-dy + ry) * psf_w + (-dx + rx)]; });
 
     k_noalloc_setup<<<1, 256, 0, stream>>>(t, s);
     cudaError_t e = cudaGetLastError();

@@ -77,6 +77,9 @@ struct eecmg_plan_s {
     static constexpr int NVEC = 9;
     float* vec[NVEC] = {};              // solver vectors, each max level size
     cudaStream_t cap_stream = nullptr;
+    // the branch of the captured cascade that solves level 0 beside level 1
+    cudaStream_t side_stream = nullptr;
+    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
     cudaGraphExec_t gexec = nullptr;
     cudaStream_t last_stream = nullptr;
     eecmg::Profiler prof;
