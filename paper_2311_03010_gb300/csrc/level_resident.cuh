@@ -113,9 +113,6 @@ __device__ __forceinline__ void conv_load_res(ConvSmem<R, SEP>& S, unsigned int 
     }
 }
 
-// One convolution phase over this block's tiles: the input is u0 in global
-// memory (GLOBAL) or vector k of the cluster (ZERO: an all-zero input, no
-// loads); the epilogue gets (local index, level index, (C (*) x)(p), x(p)).
 // conv_compute on two staged tiles at once: every thread carries the outputs
 // of both tiles through the same loops (twice the independent chains while a
 // block holds one SM), with the operations of conv_compute per output.
@@ -219,17 +216,46 @@ __device__ __forceinline__ void conv_compute2(ConvSmem<R, SEP>& A, ConvSmem<R, S
     }
 }
 
+// The tile at (y0, x0) of a level in global memory into t: every load is issued
+// before the first store (one round trip instead of one per eight rows).
+__device__ __forceinline__ void load_tile(float* t, const float* x, const ResCtx& X, int y0, int x0) {
+    float v[TILE_PX / NTHREADS];
+#pragma unroll
+    for (int k = 0; k < TILE_PX / NTHREADS; ++k) {
+        const int p = threadIdx.x + k * NTHREADS, gy = y0 + p / CONV_TW, gx = x0 + p % CONV_TW;
+        v[k] = gy < X.h && gx < X.w ? __ldcg(x + (size_t)gy * X.w + gx) : 0.f;
+    }
+#pragma unroll
+    for (int k = 0; k < TILE_PX / NTHREADS; ++k) {
+        const int p = threadIdx.x + k * NTHREADS, gy = y0 + p / CONV_TW, gx = x0 + p % CONV_TW;
+        if (gy < X.h && gx < X.w) t[p] = v[k];
+    }
+}
+
 // One convolution phase over this block's tiles: the input is u0 in global
 // memory (GLOBAL) or vector k of the cluster (ZERO: an all-zero input, no
-// loads); the epilogue gets (local index, level index, (C (*) x)(p), x(p)).
+// loads); the epilogue gets (local index, level index, (C (*) x)(p), x(p), pre(p)),
+// pre a vector in global memory that those first phases read: its loads are
+// issued before the tile is convolved (in the epilogue each waited behind the
+// stores: 13 us for the first phase of a 256^2 level).
 // S[0] stages one tile at a time; with two tiles of the cluster's vector
 // both are staged (S[0], S[1]) and computed together.  Only S[0] holds taps.
 template <int R, bool SEP, bool PREC, bool ZERO, bool GLOBAL, class Epi>
 __device__ __forceinline__ void conv_phase_res(ConvSmem<R, SEP> (&S)[2], const ResCtx& X, int k,
-                                               const float* xg, Epi&& epi) {
+                                               const float* xg, const float* pre, Epi&& epi) {
     using SM = ConvSmem<R, SEP>;
     __shared__ unsigned int nbr[2][9];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    float pv[CONV_TH / 8][2] = {};
+    auto fetch_pre = [&](int y0, int x0) {
+#pragma unroll
+        for (int it = 0; it < CONV_TH / 8; ++it)
+#pragma unroll
+            for (int hf = 0; hf < 2; ++hf) {
+                const int gy = y0 + warp + 8 * it, gx = x0 + lane + 32 * hf;
+                pv[it][hf] = (ZERO || GLOBAL) && gy < X.h && gx < X.w ? __ldg(pre + (size_t)gy * X.w + gx) : 0.f;
+            }
+    };
     auto epilogue = [&](const SM& T, int lt, int y0, int x0) {
 #pragma unroll
         for (int it = 0; it < CONV_TH / 8; ++it) {
@@ -240,7 +266,7 @@ __device__ __forceinline__ void conv_phase_res(ConvSmem<R, SEP> (&S)[2], const R
                 if (gy < X.h && gx < X.w) {
                     const float z = ZERO ? 0.f : T.out[r * SM::PO + c];
                     const float ctr = ZERO ? 0.f : T.in[SM::at(r + R, c + R)];
-                    epi(lt * TILE_PX + r * CONV_TW + c, (size_t)gy * X.w + gx, z, ctr);
+                    epi(lt * TILE_PX + r * CONV_TW + c, (size_t)gy * X.w + gx, z, ctr, pv[it][hf]);
                 }
             }
         }
@@ -261,6 +287,7 @@ __device__ __forceinline__ void conv_phase_res(ConvSmem<R, SEP> (&S)[2], const R
         const int t = t0 + lt;
         if (t >= X.ntiles) break;
         const int y0 = (t / X.tiles_x) * CONV_TH, x0 = (t % X.tiles_x) * CONV_TW;
+        fetch_pre(y0, x0);
         if (!ZERO) {
             if (GLOBAL)
                 conv_load<R, SEP, true, float>(S[0], xg, X.h, X.w, y0, x0);
@@ -338,10 +365,7 @@ __device__ __forceinline__ void mr2_res_body(ConvSmem<R, SEP> (&S)[2], PsdSmem& 
                 const int t = X.bid * X.T + lt;
                 if (t >= X.ntiles) break;
                 const int y0 = (t / X.tiles_x) * CONV_TH, x0 = (t % X.tiles_x) * CONV_TW;
-                for (int p = threadIdx.x; p < TILE_PX; p += NTHREADS) {
-                    const int gy = y0 + p / CONV_TW, gx = x0 + p % CONV_TW;
-                    if (gy < X.h && gx < X.w) u[lt * TILE_PX + p] = __ldcg(J.u + (size_t)gy * X.w + gx);
-                }
+                load_tile(u + lt * TILE_PX, J.u, X, y0, x0);
             }
         }
         __syncthreads();
@@ -354,8 +378,7 @@ __device__ __forceinline__ void mr2_res_body(ConvSmem<R, SEP> (&S)[2], PsdSmem& 
         float a0 = 0.f, a1 = 0.f;
         float* rv_ = X.vec(VR);
         const bool zs = J.zero_start != 0;
-        auto epi = [&](int li, size_t gi, float z, float) {
-            const float gv = __ldg(J.g + gi);
+        auto epi = [&](int li, size_t gi, float z, float, float gv) {
             const float rv = gv - z;
             rv_[li] = rv;
             if (zs) J.u[gi] = 0.f;  // the zero start, in global memory for an early return
@@ -363,9 +386,9 @@ __device__ __forceinline__ void mr2_res_body(ConvSmem<R, SEP> (&S)[2], PsdSmem& 
             a1 = fmaf(gv, gv, a1);
         };
         if (J.zero_start)
-            conv_phase_res<R, SEP, PREC, true, true>(S, X, 0, J.u, epi);
+            conv_phase_res<R, SEP, PREC, true, true>(S, X, 0, J.u, J.g, epi);
         else
-            conv_phase_res<R, SEP, PREC, false, true>(S, X, 0, J.u, epi);
+            conv_phase_res<R, SEP, PREC, false, true>(S, X, 0, J.u, J.g, epi);
         float v[2] = {a0, a1};
         const double ct2 = J.conv_tol2, d2 = J.disc2;
         const int ear = J.early;
@@ -384,8 +407,8 @@ __device__ __forceinline__ void mr2_res_body(ConvSmem<R, SEP> (&S)[2], PsdSmem& 
     {
         float a0 = 0.f, a1 = 0.f;
         float* v1 = X.vec(VV + 1);
-        conv_phase_res<R, SEP, PREC, false, false>(S, X, VR, nullptr,
-                                                   [&](int li, size_t, float z, float ctr) {
+        conv_phase_res<R, SEP, PREC, false, false>(S, X, VR, nullptr, nullptr,
+                                                   [&](int li, size_t, float z, float ctr, float) {
                                                        v1[li] = z;
                                                        a0 = fmaf(z, z, a0);
                                                        a1 = fmaf(z, ctr, a1);
@@ -406,8 +429,8 @@ __device__ __forceinline__ void mr2_res_body(ConvSmem<R, SEP> (&S)[2], PsdSmem& 
             const float scale = vldf(&sc->f_scale);
             float a0 = 0.f;
             float* aw = X.vec(VAW + sk);
-            conv_phase_res<R, SEP, PREC, false, false>(S, X, VV + sk, nullptr,
-                                                       [&](int li, size_t, float z, float ctr) {
+            conv_phase_res<R, SEP, PREC, false, false>(S, X, VV + sk, nullptr, nullptr,
+                                                       [&](int li, size_t, float z, float ctr, float) {
                                                            const float hz = z * scale;
                                                            aw[li] = hz;
                                                            a0 = fmaf(hz, ctr, a0);
@@ -551,10 +574,7 @@ __device__ __forceinline__ void cgls_res_body(ConvSmem<R, SEP> (&S)[2], PsdSmem&
                 const int t = X.bid * X.T + lt;
                 if (t >= X.ntiles) break;
                 const int y0 = (t / X.tiles_x) * CONV_TH, x0 = (t % X.tiles_x) * CONV_TW;
-                for (int p = threadIdx.x; p < TILE_PX; p += NTHREADS) {
-                    const int gy = y0 + p / CONV_TW, gx = x0 + p % CONV_TW;
-                    if (gy < X.h && gx < X.w) u[lt * TILE_PX + p] = __ldcg(J.u + (size_t)gy * X.w + gx);
-                }
+                load_tile(u + lt * TILE_PX, J.u, X, y0, x0);
             }
         }
         __syncthreads();
@@ -568,8 +588,7 @@ __device__ __forceinline__ void cgls_res_body(ConvSmem<R, SEP> (&S)[2], PsdSmem&
     {  // r_0 = g - H u_0
         float a0 = 0.f, a1 = 0.f;
         const bool zs = J.zero_start != 0;
-        auto epi = [&](int li, size_t gi, float z, float) {
-            const float gv = __ldg(J.g + gi);
+        auto epi = [&](int li, size_t gi, float z, float, float gv) {
             const float rv = gv - z;
             rv_[li] = rv;
             if (zs) J.u[gi] = 0.f;  // the zero start, in global memory for an early return
@@ -577,9 +596,9 @@ __device__ __forceinline__ void cgls_res_body(ConvSmem<R, SEP> (&S)[2], PsdSmem&
             a1 = fmaf(gv, gv, a1);
         };
         if (J.zero_start)
-            conv_phase_res<R, SEP, PREC, true, true>(S, X, 0, J.u, epi);
+            conv_phase_res<R, SEP, PREC, true, true>(S, X, 0, J.u, J.g, epi);
         else
-            conv_phase_res<R, SEP, PREC, false, true>(S, X, 0, J.u, epi);
+            conv_phase_res<R, SEP, PREC, false, true>(S, X, 0, J.u, J.g, epi);
         float v[2] = {a0, a1};
         const double ct2 = J.conv_tol2, d2 = J.disc2;
         const int ear = J.early;
@@ -595,7 +614,7 @@ __device__ __forceinline__ void cgls_res_body(ConvSmem<R, SEP> (&S)[2], PsdSmem&
     __syncthreads();
     {
         float a0 = 0.f;
-        conv_phase_res<R, SEP, PREC, false, false>(S, X, CR, nullptr, [&](int li, size_t, float z, float) {
+        conv_phase_res<R, SEP, PREC, false, false>(S, X, CR, nullptr, nullptr, [&](int li, size_t, float z, float, float) {
             sv[li] = z;
             pv[li] = z;
             a0 = fmaf(z, z, a0);
@@ -611,7 +630,7 @@ __device__ __forceinline__ void cgls_res_body(ConvSmem<R, SEP> (&S)[2], PsdSmem&
         __syncthreads();
         {
             float a0 = 0.f;
-            conv_phase_res<R, SEP, PREC, false, false>(S, X, CP, nullptr, [&](int li, size_t, float z, float) {
+            conv_phase_res<R, SEP, PREC, false, false>(S, X, CP, nullptr, nullptr, [&](int li, size_t, float z, float, float) {
                 qv[li] = z;
                 a0 = fmaf(z, z, a0);
             });
@@ -639,7 +658,7 @@ __device__ __forceinline__ void cgls_res_body(ConvSmem<R, SEP> (&S)[2], PsdSmem&
         __syncthreads();
         {
             float a0 = 0.f;
-            conv_phase_res<R, SEP, PREC, false, false>(S, X, CR, nullptr, [&](int li, size_t, float z, float) {
+            conv_phase_res<R, SEP, PREC, false, false>(S, X, CR, nullptr, nullptr, [&](int li, size_t, float z, float, float) {
                 sv[li] = z;
                 a0 = fmaf(z, z, a0);
             });
