@@ -118,12 +118,15 @@ eecmg_status plan_waves(const std::vector<std::pair<eecmg_plan_s*, int>>& items,
     return EECMG_OK;
 }
 
-cudaError_t Fan::create() {
+cudaError_t Fan::add(int i) {
+    if (side[i]) return cudaSuccess;
+    cudaError_t e = join[i] ? cudaSuccess : cudaEventCreateWithFlags(&join[i], cudaEventDisableTiming);
+    return e == cudaSuccess ? cudaStreamCreateWithFlags(&side[i], cudaStreamNonBlocking) : e;
+}
+
+cudaError_t Fan::create(int n) {
     cudaError_t e = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);
-    for (int i = 0; i < SIDES && e == cudaSuccess; ++i) {
-        e = cudaStreamCreateWithFlags(&side[i], cudaStreamNonBlocking);
-        if (e == cudaSuccess) e = cudaEventCreateWithFlags(&join[i], cudaEventDisableTiming);
-    }
+    for (int i = 0; i < n && i < SIDES && e == cudaSuccess; ++i) e = add(i);
     return e;
 }
 
@@ -145,10 +148,11 @@ void Fan::begin(cudaStream_t s) {
 }
 
 cudaError_t Fan::next(cudaStream_t* out) {
-    cudaError_t e = cudaSuccess;
+    const int i = n_ % SIDES;
+    cudaError_t e = add(i);
+    if (e != cudaSuccess) return e;  // nothing forked onto it yet
     if (!forked_) e = cudaEventRecord(fork, main_);
     forked_ = true;
-    const int i = n_ % SIDES;
     if (e == cudaSuccess && n_ < SIDES) e = cudaStreamWaitEvent(side[i], fork, 0);
     ++n_;
     *out = side[i];
@@ -501,7 +505,15 @@ eecmg_status build_ctx(BatchCtx& C) {
             ok = level_shape(P->lv[l].h, P->lv[l].w, P->lv[l].rt, cg, bf).resident > 0;
         C.fork01 = C.fork01 && ok;
     }
-    if (C.fan.create() != cudaSuccess) return set_error(EECMG_ERR_CUDA, "eecmg_restore_batched: side streams");
+    size_t sides = 0;  // the most cluster waves that a step (or steps 0 and 1 together) holds
+    for (int s = 0; s < maxL; ++s) {
+        size_t k = 0;
+        for (const Wave& w : C.steps[s]) k += w.cluster > 0;
+        if (s == 0 && C.fork01)
+            for (const Wave& w : C.steps[1]) k += w.cluster > 0;
+        sides = std::max(sides, k);
+    }
+    if (C.fan.create((int)std::min<size_t>(sides, Fan::SIDES)) != cudaSuccess) return set_error(EECMG_ERR_CUDA, "eecmg_restore_batched: side streams");
     return EECMG_OK;
 }
 

@@ -44,7 +44,8 @@ struct Fan {
     static constexpr int SIDES = 8;
     cudaStream_t side[SIDES] = {};
     cudaEvent_t fork = nullptr, join[SIDES] = {};
-    cudaError_t create();
+    // n side streams at once (a capture creates none); further ones come at first use
+    cudaError_t create(int n);
     void destroy();
     // Queues a cluster launch on the next side stream; begin() forks the side streams
     // off s at their first use, end() joins those used back into s.
@@ -53,6 +54,7 @@ struct Fan {
     cudaError_t end();
 
 private:
+    cudaError_t add(int i);
     cudaStream_t main_ = nullptr;
     int n_ = 0;       // cluster launches so far
     bool forked_ = false;

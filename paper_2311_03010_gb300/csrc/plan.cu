@@ -511,6 +511,11 @@ eecmg_status cascade_enqueue(eecmg_plan_s* P, cudaStream_t s) {
 eecmg_status run_cascade(eecmg_plan_s* P, cudaStream_t s) {
     if (!P->opt.use_graph || P->prof.on) return cascade_enqueue(P, s);
     if (!P->gexec) {
+        if (coarse_pair_independent(P)) {  // the second branch (made here: plans of a batch never need it)
+            if (!P->side_stream) CK(cudaStreamCreateWithFlags(&P->side_stream, cudaStreamNonBlocking));
+            if (!P->ev_fork) CK(cudaEventCreateWithFlags(&P->ev_fork, cudaEventDisableTiming));
+            if (!P->ev_join) CK(cudaEventCreateWithFlags(&P->ev_join, cudaEventDisableTiming));
+        }
         CK(cudaStreamBeginCapture(P->cap_stream, cudaStreamCaptureModeThreadLocal));
         eecmg_status st = cascade_enqueue(P, P->cap_stream);
         cudaGraph_t graph = nullptr;
@@ -553,18 +558,11 @@ eecmg_status plan_allocate(eecmg_plan_s* P, const char* who) {
     if (e == cudaSuccess)
         e = cudaMemcpy(P->dtaps, P->htaps.data(), sizeof(Taps) * 2 * P->L, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&P->cap_stream, cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&P->side_stream, cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&P->ev_fork, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&P->ev_join, cudaEventDisableTiming);
     if (e != cudaSuccess) {
         cudaFree(P->ws);
         P->ws = nullptr;
         if (P->cap_stream) cudaStreamDestroy(P->cap_stream);
-        if (P->side_stream) cudaStreamDestroy(P->side_stream);
-        if (P->ev_fork) cudaEventDestroy(P->ev_fork);
-        if (P->ev_join) cudaEventDestroy(P->ev_join);
-        P->cap_stream = P->side_stream = nullptr;
-        P->ev_fork = P->ev_join = nullptr;
+        P->cap_stream = nullptr;
         return set_error(EECMG_ERR_CUDA, std::string(who) + ": " + cudaGetErrorString(e));
     }
     P->owns_ws = true;
