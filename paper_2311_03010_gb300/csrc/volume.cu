@@ -242,6 +242,8 @@ VolJob make_job(eecmg_vol_s* P, int l, bool transpose) {
 
 // The (tile, slice) pairs a convolution phase divides over the blocks.
 long long level_units(int d, int h, int w, const VolTaps& t) {
+    if (t.form == VF_SMALL || t.form == VF_SPARSE)  // output tiles
+        return (long long)((w + TX - 1) / TX) * ((h + TY - 1) / TY) * ((d + TZ - 1) / TZ);
     const int sy = form_rows(t.r, t.form);
     return (long long)((w + MX - 1) / MX) * ((h + sy - 1) / sy) * d;
 }
@@ -494,12 +496,20 @@ eecmg_status eecmg_vol_plan(int width, int height, int depth, int levels, const 
         delete P;
         return set_error(EECMG_ERR_CUDA, std::string("eecmg_vol_plan: ") + cudaGetErrorString(e));
     }
+    // few slices per block to march (two blocks per SM): tiles (62 x 146 x 25, r = 3, 1.2 slices
+    // a block: solve 121 us marched, 83 us in tiles; 256^3, 33 slices a block: 46 against 113 us
+    // a convolution)
+    for (int l = 0; l < L; ++l)
+        for (VolTaps* t : {&P->taps[l], &P->tapsT[l]})
+            if (t->form == VF_SEP && level_units(P->ds[l], P->hs[l], P->ws[l], *t) < 2LL * t->r * 2 * P->sms)
+                t->form = VF_SMALL;
     P->grid.resize(L);
     int maxgrid = 1;
     for (int l = 0; l < L; ++l) {
         // the attribute belongs to the kernel, which plans of every form share
         const int r = P->taps[l].r;
-        const size_t most = std::max(form_bytes(r, VF_SEP), std::max(form_bytes(r, VF_DENSE), form_bytes(r, VF_SPARSE)));
+        size_t most = 0;
+        for (int f : {VF_SEP, VF_DENSE, VF_SPARSE, VF_SMALL}) most = std::max(most, form_bytes(r, f));
         const size_t smem = form_bytes(r, P->taps[l].form);
         e = cudaFuncSetAttribute(vol_kernels().solve[r], cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)most);

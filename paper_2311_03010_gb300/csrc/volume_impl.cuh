@@ -17,13 +17,14 @@ namespace vol {
 constexpr int VR = EECMG_VOL_MAX_RADIUS;
 constexpr int VK = 2 * VR + 1;
 constexpr int MX = 64;                  // columns of a marched tile
-constexpr int TX = 32, TY = 8, TZ = 8;  // sparse form: output tile (columns, rows, slices)
+constexpr int TX = 32, TY = 8, TZ = 8;  // small and sparse forms: output tile (columns, rows, slices)
 
 // How a level's PSF is applied (fixed by the planner from its taps).
 enum VolForm : int {
     VF_SEP = 0,     // an outer product of three factors: three 1-D passes
     VF_DENSE = 1,   // rows of 2 r + 1 taps for every (slice, row) offset that has one
     VF_SPARSE = 2,  // a list of taps
+    VF_SMALL = 3,   // as VF_SEP, on a level with few slices per block to march
 };
 
 // Taps of one level in correlation form, y(v) = sum_d C(d) x(v + d), C(d) = K(-d),
@@ -31,7 +32,7 @@ enum VolForm : int {
 struct VolTaps {
     int r;
     int form;                      // VolForm
-    float cz[VK], cy[VK], cx[VK];  // VF_SEP: factors, index d + r
+    float cz[VK], cy[VK], cx[VK];  // VF_SEP, VF_SMALL: factors, index d + r
     int ntap;                      // else: taps in the job's tap list
 };
 
@@ -524,11 +525,159 @@ __device__ __forceinline__ void sparse_phase(const VolJob& J, const float* __res
     }
 }
 
+// VF_SMALL: 8 x 8 x 32 output tiles, the next tile's window (zero outside the
+// volume) in flight by cp.async while this one is convolved: slices over every
+// staged (row, column) into B, rows into C (over the window's own buffer),
+// columns over C.  A marching block repeats 2 r slices whatever its share, so below
+// 2 r slices a block the tiles are faster (GB300, 45 x 70 x 61, r = 2: 4.4 us a
+// convolution against 5.9 us; 128^3, 4.2 slices a block, 11.2 against 10.9 us).
+template <int R>
+struct SmallTile {
+    static constexpr int PADX = (R + 3) / 4 * 4, X0 = PADX - R;
+    static constexpr int NZ = TZ + 2 * R, NY = TY + 2 * R, AX = TX + 2 * PADX;
+    static constexpr int IN = NZ * NY * AX, MID = TZ * NY * AX;
+    static constexpr size_t bytes = sizeof(float) * (2 * (size_t)IN + MID);
+};
+template <int R>
+__device__ __forceinline__ void stage_small(const VolJob& J, const float* __restrict__ x, int x0, int y0, int z0, float* A,
+                                            bool vec) {
+    using S = SmallTile<R>;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned int base = smem_u32(A);
+    if (vec) {
+        constexpr int CH = S::AX / 4, RPW = 32 / CH, ROWS = S::NZ * S::NY;  // chunks per row, rows per warp
+        const int sub = lane / CH, c = lane - sub * CH;
+        for (int r0 = warp * RPW; r0 < ROWS; r0 += (NTHREADS / 32) * RPW) {
+            const int row = r0 + sub;
+            if (sub >= RPW || row >= ROWS) continue;
+            const int gz = z0 - R + row / S::NY, gy = y0 - R + row % S::NY, gx = x0 - S::PADX + 4 * c;
+            const bool in = gz >= 0 && gz < J.d && gy >= 0 && gy < J.h && gx >= 0 && gx < J.w;
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(
+                             base + 4u * (unsigned int)(row * S::AX + 4 * c)),
+                         "l"(in ? x + ((long long)gz * J.h + gy) * J.w + gx : x), "r"(in ? 16 : 0)
+                         : "memory");
+        }
+    } else {
+        for (int row = warp; row < S::NZ * S::NY; row += NTHREADS / 32) {
+            const int gz = z0 - R + row / S::NY, gy = y0 - R + row % S::NY;
+            const bool rin = gz >= 0 && gz < J.d && gy >= 0 && gy < J.h;
+            const float* src = x + ((long long)(rin ? gz : 0) * J.h + (rin ? gy : 0)) * J.w;
+#pragma unroll
+            for (int c = lane; c < S::AX; c += 32) {
+                const int gx = x0 - S::PADX + c;
+                const bool in = rin && gx >= 0 && gx < J.w;
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(
+                                 base + 4u * (unsigned int)(row * S::AX + c)),
+                             "l"(in ? src + gx : x), "r"(in ? 4 : 0)
+                             : "memory");
+            }
+        }
+    }
+    commit_copies();
+}
+template <int R>
+__device__ __forceinline__ void small_phase(const VolJob& J, const float* __restrict__ x, float* sm, const EpiArgs& E,
+                                            DF (&acc)[2]) {
+    using S = SmallTile<R>;
+    const VolTaps& K = J.taps;
+    const int ntx = (J.w + TX - 1) / TX, nty = (J.h + TY - 1) / TY;
+    const int ntiles = ntx * nty * ((J.d + TZ - 1) / TZ), nb = gridDim.x;
+    const int xo = threadIdx.x & 31, yo = threadIdx.x >> 5;
+    const bool vec = (J.w & 3) == 0 && aligned16(x, nullptr, nullptr);
+    float* B = sm + 2 * S::IN;
+    int t = blockIdx.x, buf = 0;
+    if (t >= ntiles) return;  // the whole block
+    auto origin = [&](int k, int& x0, int& y0, int& z0) {
+        x0 = (k % ntx) * TX;
+        y0 = ((k / ntx) % nty) * TY;
+        z0 = (k / ntx / nty) * TZ;
+    };
+    int x0, y0, z0;
+    origin(t, x0, y0, z0);
+    stage_small<R>(J, x, x0, y0, z0, sm, vec);
+    for (; t < ntiles; t += nb, buf ^= 1) {
+        origin(t, x0, y0, z0);
+        if (t + nb < ntiles) {
+            int x1, y1, z1;
+            origin(t + nb, x1, y1, z1);
+            stage_small<R>(J, x, x1, y1, z1, sm + (buf ^ 1) * S::IN, vec);
+            wait_copies<1>();
+        } else {
+            wait_copies<0>();
+        }
+        __syncthreads();
+        float* A = sm + buf * S::IN;
+        const int gx = x0 + xo, gy = y0 + yo;
+        const bool in = gy < J.h && gx < J.w;
+        // the epilogue's operands, fetched before the passes
+        float pa[TZ], pb[TZ];
+#pragma unroll
+        for (int z = 0; z < TZ; ++z) {
+            const size_t i = ((size_t)(z0 + z) * J.h + gy) * J.w + gx;
+            const bool ok = in && z0 + z < J.d;
+            pa[z] = ok && E.a ? __ldcg(E.a + i) : 0.f;
+            pb[z] = ok && E.b ? __ldcg(E.b + i) : 0.f;
+        }
+        constexpr int COLS = S::NY * S::AX;
+        for (int c = threadIdx.x; c < COLS; c += NTHREADS) {
+            float win[S::NZ];
+#pragma unroll
+            for (int z = 0; z < S::NZ; ++z) win[z] = A[z * COLS + c];
+#pragma unroll
+            for (int z = 0; z < TZ; ++z) {
+                float s = 0.f;
+#pragma unroll
+                for (int o = 0; o <= 2 * R; ++o) s = fmaf(K.cz[o], win[z + o], s);
+                B[z * COLS + c] = s;
+            }
+        }
+        __syncthreads();
+        constexpr int COLS2 = TZ * S::AX;
+        for (int c = threadIdx.x; c < COLS2; c += NTHREADS) {
+            const int z = c / S::AX, xx = c - z * S::AX;
+            const float* b = B + z * COLS + xx;
+            float win[S::NY];
+#pragma unroll
+            for (int y = 0; y < S::NY; ++y) win[y] = b[y * S::AX];
+#pragma unroll
+            for (int y = 0; y < TY; ++y) {
+                float s = 0.f;
+#pragma unroll
+                for (int p = 0; p <= 2 * R; ++p) s = fmaf(K.cy[p], win[y + p], s);
+                A[(z * TY + y) * S::AX + xx] = s;
+            }
+        }
+        __syncthreads();
+        float s[TZ];
+#pragma unroll
+        for (int z = 0; z < TZ; ++z) {
+            s[z] = 0.f;
+            const float* c = A + (z * TY + yo) * S::AX + S::X0 + xo;
+#pragma unroll
+            for (int q = 0; q <= 2 * R; ++q) s[z] = fmaf(K.cx[q], c[q], s[z]);
+        }
+        if (in) {
+#pragma unroll
+            for (int z = 0; z < TZ; ++z) {
+                if (z0 + z >= J.d) break;
+                float sa = 0.f, sb = 0.f;
+                epilogue4(E, ((size_t)(z0 + z) * J.h + gy) * J.w + gx, 1, false, make_float4(s[z], 0.f, 0.f, 0.f),
+                          make_float4(pa[z], 0.f, 0.f, 0.f), make_float4(pb[z], 0.f, 0.f, 0.f), sa, sb);
+                acc_add(acc[0], sa);
+                acc_add(acc[1], sb);
+            }
+        }
+        __syncthreads();  // the buffers are restaged after this
+    }
+}
+
 template <int R>
 __device__ __forceinline__ void conv_phase(const VolJob& J, const float* __restrict__ x, float* sm, const EpiArgs& E,
                                            DF (&acc)[2]) {
     if (J.taps.form == VF_SEP)
         sep_phase<R>(J, x, sm, E, acc);
+    else if (J.taps.form == VF_SMALL)
+        small_phase<R>(J, x, sm, E, acc);
     else if (J.taps.form == VF_DENSE)
         dense_phase<R>(J, x, sm, E, acc);
     else
@@ -728,7 +877,7 @@ __global__ void __launch_bounds__(NTHREADS, 2) k_vol_apply(const __grid_constant
 // tiles whose slices a phase divides over the blocks.
 template <int R>
 constexpr size_t vol_smem(int form) {
-    return form == VF_SPARSE ? SparseTile<R>::bytes : March<R>::bytes(form);
+    return form == VF_SPARSE ? SparseTile<R>::bytes : form == VF_SMALL ? SmallTile<R>::bytes : March<R>::bytes(form);
 }
 template <int R>
 constexpr int vol_tile_rows(int form) {
