@@ -695,7 +695,7 @@ __device__ __forceinline__ void conv_phase(const VolJob& J, const float* __restr
 // to the first, so that a phase finds the end of what the phase before streamed still
 // in L2 (the update after the new directions), and the first output streaming (u, not
 // read again before the next update): 256^3, 3 iterations, 3.09 -> 3.03 GB of DRAM traffic
-// by the order alone.
+// by the order alone, 2.98 with u and g streamed.
 template <bool REV, int NL, int NS, class F>
 __device__ __forceinline__ void vec_phase(long long n4, long long gtid, long long gstr,
                                           const float4* const (&in)[NL], float4* const (&out)[NS],
