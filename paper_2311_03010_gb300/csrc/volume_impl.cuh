@@ -57,11 +57,11 @@ struct VolJob {
     double* out;        // [0] iterations, [1] ||r||^2, [2] stop reason
 };
 
-// Per-block replica of the solve's scalars (identical in every block), as
-// double-float pairs: on GB300 a dependent FP64 operation takes 66 cycles, and the
-// divisions and roots of these updates took 4-6 us of every phase in FP64.
+// Per-block replica of the solve's scalars (identical in every block), in FP64.  A
+// dependent FP64 operation takes 66 cycles on GB300, so a phase takes at most one
+// quotient (its two are independent) and no root: the stop test is on ||r||^2.
 struct VolScal {
-    DF rr, qq, qqp, qqn, lim2;
+    double rr, qq, qqp, qqn, lim2;
     float a, b1, b2;
     int k, done;
 };
@@ -729,7 +729,7 @@ __device__ __forceinline__ void vec_phase(long long n4, long long gtid, long lon
 
 // ------------------------------------------------------------- level solve
 
-__device__ __forceinline__ bool df_pos_finite(DF x) { return x.hi > 0.f && df_finite(x); }
+__device__ __forceinline__ bool pos_finite(double x) { return x > 0.0 && isfinite(x); }
 
 // MR-II (the three-term recurrence of the oracle's level smoother):
 //   r0 = g - H u0;  p1 = H r0, q1 = H p1, a = <r,q>/<q,q>, u += a p, r -= a q;
@@ -834,33 +834,27 @@ __global__ void __launch_bounds__(NTHREADS, 2) k_vol_mr2(const __grid_constant__
             conv_phase<R>(J, x, sm, E, acc);
         }
         ok = grid_reduce_df<2>(acc, J.partials, J.gs, nb, bid, phase++, [&](const DF (&t)[2]) {
+            const double t0 = df_to_double(t[0]), t1 = df_to_double(t[1]);
             if (kind <= PH_R0) {
-                S.rr = t[0];
+                S.rr = t0;
                 S.k = 0;
                 // the limit of both rules, formed once (off the later phases' path)
-                const double gg = df_to_double(t[1]);
-                const double l1 = J.conv_tol * J.conv_tol * gg, l2 = J.stop_tol * J.stop_tol * (double)J.n;
-                S.lim2 = df_from_double(l1 > l2 ? l1 : l2);
-                const bool rule = J.stop_tol > 0.0 || J.conv_tol > 0.0;
-                if (!rule) S.lim2 = DF{-1.f, 0.f};
-                S.done = (J.m <= 0 || df_le(S.rr, S.lim2)) ? 1 : 0;
-            } else if (kind == PH_Q1) {
-                S.done = df_pos_finite(t[0]) ? 0 : 2;
-                S.qqn = t[0];
-                S.a = df_div(t[1], t[0]).hi;
+                S.lim2 = fmax(J.conv_tol > 0.0 ? J.conv_tol * J.conv_tol * t1 : -1.0,
+                              J.stop_tol > 0.0 ? J.stop_tol * J.stop_tol * (double)J.n : -1.0);
+                S.done = (J.m <= 0 || t0 <= S.lim2) ? 1 : 0;
+            } else if (kind == PH_Q1 || kind == PH_DIR) {
+                S.done = pos_finite(t0) ? 0 : 2;
+                S.qqn = t0;
+                S.a = (float)(t1 / t0);
             } else if (kind == PH_Z) {
-                S.b1 = df_div(t[0], S.qq).hi;
-                S.b2 = k >= 2 ? df_div(t[1], S.qqp).hi : 0.f;
-            } else if (kind == PH_DIR) {
-                S.done = df_pos_finite(t[0]) ? 0 : 2;
-                S.qqn = t[0];
-                S.a = df_div(t[1], t[0]).hi;
+                S.b1 = (float)(t0 / S.qq);
+                S.b2 = k >= 2 ? (float)(t1 / S.qqp) : 0.f;
             } else if (kind == PH_UPD) {
-                S.rr = t[0];
+                S.rr = t0;
                 S.qqp = S.qq;
                 S.qq = S.qqn;
                 S.k = k + 1;
-                S.done = (S.k >= J.m || df_le(S.rr, S.lim2)) ? 1 : 0;
+                S.done = (S.k >= J.m || t0 <= S.lim2) ? 1 : 0;
             }
         });
         if (!ok || S.done) break;
@@ -872,7 +866,7 @@ __global__ void __launch_bounds__(NTHREADS, 2) k_vol_mr2(const __grid_constant__
     }
     if (bid == 0 && threadIdx.x == 0) {
         J.out[0] = S.k;
-        J.out[1] = df_to_double(S.rr);
+        J.out[1] = S.rr;
         J.out[2] = ok ? S.done : -1;
     }
     grid_exit(J.gs, nb);
