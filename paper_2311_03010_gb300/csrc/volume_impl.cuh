@@ -107,25 +107,46 @@ __device__ __forceinline__ float4 ld_quad(const float* p, size_t i, int nv, bool
     return r;
 }
 
-// Four outputs of a row at element i, of which nv (1..4) lie in the volume; their
-// products are added to sa, sb.
+// The products of four pairs into a compensated sum, one at a time: a sum of them in
+// plain FP32 would lose what the compensation keeps.
+__device__ __forceinline__ void acc_dot(DF& s, float4 a, float4 b) {
+    acc_add(s, a.x * b.x);
+    acc_add(s, a.y * b.y);
+    acc_add(s, a.z * b.z);
+    acc_add(s, a.w * b.w);
+}
+__device__ __forceinline__ void acc_dot(DF& s, float a, float b) { acc_add(s, a * b); }
+__device__ __forceinline__ float sub(float a, float b) { return a - b; }
+__device__ __forceinline__ float4 sub(float4 a, float4 b) {
+    return make_float4(a.x - b.x, a.y - b.y, a.z - b.z, a.w - b.w);
+}
+
+// What a phase stores for one (T = float) or four outputs of a row, and their products
+// into the phase's sums.
+template <class T>
+__device__ __forceinline__ T epilogue(const EpiArgs& E, T hx, T a, T b, DF (&acc)[2]) {
+    if (E.mode == VE_RESID) {
+        const T o = sub(a, hx);
+        acc_dot(acc[0], o, o);
+        acc_dot(acc[1], a, a);
+        return o;
+    }
+    if (E.mode == VE_Q1) {
+        acc_dot(acc[0], hx, hx);
+        acc_dot(acc[1], a, hx);
+    } else if (E.mode == VE_Z) {
+        acc_dot(acc[0], a, hx);
+        acc_dot(acc[1], b, hx);
+    }
+    return hx;
+}
+// Four outputs of a row at element i, of which nv (1..4) lie in the volume.
 __device__ __forceinline__ void epilogue4(const EpiArgs& E, size_t i, int nv, bool vec, float4 hx, float4 a,
-                                          float4 b, float& sa, float& sb) {
+                                          float4 b, DF (&acc)[2]) {
     if (nv < 4) hx.w = a.w = 0.f;
     if (nv < 3) hx.z = a.z = 0.f;
     if (nv < 2) hx.y = a.y = 0.f;
-    float4 o = hx;
-    if (E.mode == VE_RESID) {
-        o = make_float4(a.x - hx.x, a.y - hx.y, a.z - hx.z, a.w - hx.w);
-        sa = dot4(o, o, sa);
-        sb = dot4(a, a, sb);
-    } else if (E.mode == VE_Q1) {
-        sa = dot4(hx, hx, sa);
-        sb = dot4(a, hx, sb);
-    } else if (E.mode == VE_Z) {
-        sa = dot4(a, hx, sa);
-        sb = dot4(b, hx, sb);
-    }
+    const float4 o = epilogue(E, hx, a, b, acc);
     if (vec) {
         *reinterpret_cast<float4*>(E.out + i) = o;
     } else {
@@ -306,7 +327,6 @@ __device__ __forceinline__ void sep_phase(const VolJob& J, const float* __restri
             const int b = slot & 1;
             if (emit && main) {  // columns pass
                 const float4* v = reinterpret_cast<const float4*>(V + (b ^ 1) * M::V) + g * RPT * QX + q;
-                float sa = 0.f, sb = 0.f;
 #pragma unroll
                 for (int i = 0; i < RPT; ++i) {
                     float w[4 * (2 * HQ + 1)];
@@ -325,10 +345,8 @@ __device__ __forceinline__ void sep_phase(const VolJob& J, const float* __restri
                         for (int c = 0; c < 4; ++c) o[c] = fmaf(J.taps.cx[k], w[M::PADX - R + c + k], o[c]);
                     if (nv[i] > 0)
                         epilogue4(E, at + (size_t)(i * J.w), nv[i], vec, make_float4(o[0], o[1], o[2], o[3]),
-                                  pa[i], pb[i], sa, sb);
+                                  pa[i], pb[i], acc);
                 }
-                acc_add(acc[0], sa);
-                acc_add(acc[1], sb);
             }
             if (emit) at += sl;
             if (s < s_end && work) {  // rows pass, then along the slices
@@ -455,12 +473,7 @@ __device__ __forceinline__ void dense_phase(const VolJob& J, const float* __rest
                     }
                 }
             }
-            if (emit) {
-                float sa = 0.f, sb = 0.f;
-                epilogue4(E, at, nv, vec, part[0], pa, pb, sa, sb);
-                acc_add(acc[0], sa);
-                acc_add(acc[1], sb);
-            }
+            if (emit) epilogue4(E, at, nv, vec, part[0], pa, pb, acc);
 #pragma unroll
             for (int k = 0; k < 2 * R; ++k) part[k] = part[k + 1];
             part[2 * R] = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -518,12 +531,7 @@ __device__ __forceinline__ void sparse_phase(const VolJob& J, const float* __res
             for (int z = 0; z < TZ; ++z) {
                 if (z0 + z >= J.d) break;
                 const size_t i = ((size_t)(z0 + z) * J.h + gy) * J.w + gx;
-                const float4 va = make_float4(E.a ? __ldcg(E.a + i) : 0.f, 0.f, 0.f, 0.f);
-                const float4 vb = make_float4(E.b ? __ldcg(E.b + i) : 0.f, 0.f, 0.f, 0.f);
-                float sa = 0.f, sb = 0.f;
-                epilogue4(E, i, 1, false, make_float4(s[z], 0.f, 0.f, 0.f), va, vb, sa, sb);
-                acc_add(acc[0], sa);
-                acc_add(acc[1], sb);
+                E.out[i] = epilogue(E, s[z], E.a ? __ldcg(E.a + i) : 0.f, E.b ? __ldcg(E.b + i) : 0.f, acc);
             }
         }
     }
@@ -664,11 +672,7 @@ __device__ __forceinline__ void small_phase(const VolJob& J, const float* __rest
 #pragma unroll
             for (int z = 0; z < TZ; ++z) {
                 if (z0 + z >= J.d) break;
-                float sa = 0.f, sb = 0.f;
-                epilogue4(E, ((size_t)(z0 + z) * J.h + gy) * J.w + gx, 1, false, make_float4(s[z], 0.f, 0.f, 0.f),
-                          make_float4(pa[z], 0.f, 0.f, 0.f), make_float4(pb[z], 0.f, 0.f, 0.f), sa, sb);
-                acc_add(acc[0], sa);
-                acc_add(acc[1], sb);
+                E.out[((size_t)(z0 + z) * J.h + gy) * J.w + gx] = epilogue(E, s[z], pa[z], pb[z], acc);
             }
         }
         __syncthreads();  // the buffers are restaged after this
