@@ -353,8 +353,8 @@ __global__ void __launch_bounds__(16 * DY) k_vol_pm_c(const float* __restrict__ 
         row6(s, P, uc, r);
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
-            const float gx = r[k + 2] - r[k], gy = ss[k] - nn[k], gz = un[k] - ub[k];  // twice the gradient
-            o[k] = rcp_ftz(fmaf(fmaf(gz, gz, fmaf(gx, gx, gy * gy)), 0.25f * ik2, 1.f));
+            const float gx = 0.5f * (r[k + 2] - r[k]), gy = 0.5f * (ss[k] - nn[k]), gz = 0.5f * (un[k] - ub[k]);
+            o[k] = rcp_ftz(fmaf(fmaf(gz, gz, fmaf(gx, gx, gy * gy)), ik2, 1.f));
             ub[k] = uc[k];
             uc[k] = un[k];
         }
