@@ -399,6 +399,31 @@ struct VecIO<__nv_bfloat16> {
     }
 };
 
+// 2^x, the hardware's approximation (2 ulp), subnormal results kept.
+__device__ __forceinline__ float ex2_approx(float x) {
+    float y;
+    asm("ex2.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+// 1/x, correctly rounded for 2^-30 <= x < 2^30 (NaN for NaN): the hardware's approximation and
+// one Newton step whose residual an FMA forms exactly (Markstein, "Computation of
+// elementary functions on the IBM RISC System/6000 processor", 1990).  Compared with
+// __frcp_rn on every float of that range: none differs.  The rounded intrinsic itself
+// checks its range with a branch, which doubled the time of the fused level start.
+__device__ __forceinline__ float recip(float x) {
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return __fmaf_rn(y, __fmaf_rn(-x, y, 1.f), y);
+}
+// The same for every x >= 1: results below 2^-126 are the hardware's (1 ulp), 0 for infinity.
+__device__ __forceinline__ float recip_ge1(float x) {
+    float y;
+    asm("rcp.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
+    const float r = __fmaf_rn(y, __fmaf_rn(-x, y, 1.f), y);
+    return x < 0x1p126f ? r : y;
+}
+constexpr float SQRT_LOG2E = 1.2011224087864498f;  // exp(-(s v)^2) = 2^-(SQRT_LOG2E s v)^2
+
 __device__ __forceinline__ float dot4(float4 a, float4 b, float acc) {
     acc = fmaf(a.x, b.x, acc);
     acc = fmaf(a.y, b.y, acc);

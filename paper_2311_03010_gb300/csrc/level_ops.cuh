@@ -51,20 +51,6 @@ __device__ __forceinline__ float pi_at(const float* __restrict__ u1, int w1,
 static __constant__ float c_qw[4][3] = {
     {1.f, 0.f, 0.f}, {0.375f, 0.75f, -0.125f}, {0.f, 1.f, 0.f}, {-0.125f, 0.75f, 0.375f}};
 
-// MUFU approximations with subnormal results flushed (each about 1 ulp).  In
-// S a weight below 2^-126 adds nothing to sums of at least 1, the reciprocals'
-// arguments are kept away from zero, and no decision needs a correctly rounded
-// value (see the cut in s_value).
-__device__ __forceinline__ float ex2_ftz(float x) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-__device__ __forceinline__ float rcp_ftz(float x) {
-    float y;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
 // S: weighted least-squares plane fit over the in-image 3 x 3 neighbourhood
 // with weights exp(-(scale * (u_c - u_nb))^2) (Eqs. 18-19), output the fitted
 // constant.  Solved in centred form: with W, the weighted means (sb, tb, vb)
@@ -77,10 +63,10 @@ __device__ __forceinline__ float rcp_ftz(float x) {
 
 // exp(-(scale v)^2) from ks = scale sqrt(log2 e): the weight of a pair of
 // neighbours; it does not depend on which of the two is the centre.
-__device__ __forceinline__ float s_scale_ks(float scale) { return __fmul_rn(scale, 1.2011224087864498f); }
+__device__ __forceinline__ float s_scale_ks(float scale) { return __fmul_rn(scale, SQRT_LOG2E); }
 __device__ __forceinline__ float s_weight(float v, float ks) {
     const float t = __fmul_rn(v, ks);
-    return ex2_ftz(__fmul_rn(t, -t));
+    return ex2_approx(__fmul_rn(t, -t));
 }
 // One row of three neighbours (columns -1, 0, 1): weights l, c, r, the
 // products weight x v, and their sums.
@@ -107,7 +93,7 @@ __device__ __forceinline__ float s_value(float uc, const SRow& N, const SRow& P,
     const float cvm = __fadd_rn(__fadd_rn(N.lv, dv), P.lv), cvp = __fadd_rn(__fadd_rn(N.rv, fv), P.rv);
     const float rtv = __fadd_rn(cvp, -cvm);
     const float sv = __fadd_rn(__fadd_rn(N.sumv, P.sumv), __fadd_rn(dv, fv));
-    const float iw = rcp_ftz(W);  // 1 <= W <= 9
+    const float iw = recip(W);  // 1 <= W <= 9
     const float so = __fmul_rn(sb, iw), to = __fmul_rn(tb, iw), vb = __fmul_rn(sv, iw);
     const float css = __fmaf_rn(-so, sb, mss), cst = __fmaf_rn(-so, tb, mst), ctt = __fmaf_rn(-to, tb, mtt);
     const float csv = __fmaf_rn(-vb, sb, rsv), ctv = __fmaf_rn(-vb, tb, rtv);
@@ -120,10 +106,10 @@ __device__ __forceinline__ float s_value(float uc, const SRow& N, const SRow& P,
     // small projections loses nothing to cancellation (measured against 64 bits on noisy
     // images: 3.0e-8 relative, as the eigenvector form).
     const float thr = __fmul_rn(1e-6f, W);
-    const float r0 = css > thr ? rcp_ftz(css) : 0.f;
+    const float r0 = css > thr ? recip(css) : 0.f;
     const float l = __fmul_rn(cst, r0);
     const float d1 = __fmaf_rn(-l, cst, ctt), c1 = __fmaf_rn(-l, csv, ctv), o1 = __fmaf_rn(-l, so, to);
-    const float r1 = d1 > thr ? rcp_ftz(d1) : 0.f;
+    const float r1 = d1 > thr ? recip(d1) : 0.f;
     const float g = __fmaf_rn(__fmul_rn(csv, so), r0, __fmul_rn(__fmul_rn(c1, o1), r1));
     return __fadd_rn(__fadd_rn(uc, vb), -g);
 }
@@ -150,7 +136,7 @@ __device__ __forceinline__ float smooth_value_rd(Rd rd, int h, int w, float scal
 // neighbour replaced by the centre value).
 __device__ __forceinline__ float pm_c_value(float ue, float uw, float us, float un, float inv_k2) {
     const float gx = __fmul_rn(0.5f, __fadd_rn(ue, -uw)), gy = __fmul_rn(0.5f, __fadd_rn(us, -un));
-    return rcp_ftz(__fmaf_rn(__fmaf_rn(gx, gx, __fmul_rn(gy, gy)), inv_k2, 1.f));
+    return recip_ge1(__fmaf_rn(__fmaf_rn(gx, gx, __fmul_rn(gy, gy)), inv_k2, 1.f));
 }
 // the flux from b into a (the flux from a into b is its negative)
 __device__ __forceinline__ float pm_flux(float ca, float cb, float ua, float ub) {

@@ -7,11 +7,12 @@
 // slices, so that what a slice contributes to its neighbours is formed once
 // and kept in registers; in-slice neighbours come from shared-memory planes.
 // GB300 at 256^3, one voxel per thread before -> now: Pi (128^3) 19 -> 10 us, P
-// 206 -> 17 us (its taps came from a per-lane constant index), S 825 -> 192 us, D
+// 206 -> 17 us (its taps came from a per-lane constant index), S 825 -> 257 us, D
 // 140 -> 64 us (134 + 201 MB: at the memory's rate).
 #include <algorithm>
 #include <cstdint>
 
+#include "common.cuh"
 #include "volume_start.hpp"
 
 namespace eecmg {
@@ -20,17 +21,6 @@ namespace vol {
 namespace {
 
 constexpr int SMS = 152;
-
-__device__ __forceinline__ float ex2_ftz(float x) {
-    float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
-__device__ __forceinline__ float rcp_ftz(float x) {
-    float y;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
 
 // Slices per block of a marching kernel: enough blocks for six per SM, between
 // lo (each block repeats two slices' work) and 32.
@@ -138,7 +128,7 @@ __device__ __forceinline__ Plane plane_sums(const float (&p)[9], float uc, float
             const bool ctr = MID && s == 1 && t == 1;
             v[t] = ctr ? 0.f : p[3 * s + t] - uc;
             const float e = v[t] * ks;
-            wt[t] = ctr ? 0.f : ex2_ftz(-e * e);
+            wt[t] = ctr ? 0.f : ex2_approx(-e * e);
             if (EDGE && !((in >> (3 * s + t)) & 1u)) wt[t] = 0.f;
         }
         wl[s] = wt[2] - wt[0];          // first moment along the row
@@ -174,27 +164,27 @@ __device__ __forceinline__ float fit_value(float uc, const Plane& T, const Plane
     const float m11 = (T.wss + B.wss) + M.wss, m22 = (T.wtt + B.wtt) + M.wtt, m12 = (T.wst + B.wst) + M.wst;
     const float m01 = B.ws - T.ws, m02 = B.wt - T.wt;
     const float c0 = B.v - T.v, c1 = (T.vs + B.vs) + M.vs, c2 = (T.vt + B.vt) + M.vt, sv = (T.v + B.v) + M.v;
-    const float iw = rcp_ftz(W), b0 = o0 * iw, b1 = o1 * iw, b2 = o2 * iw, vb = sv * iw, thr = 1e-6f * W;
+    const float iw = recip(W), b0 = o0 * iw, b1 = o1 * iw, b2 = o2 * iw, vb = sv * iw, thr = 1e-6f * W;
     const float a00 = fmaf(-b0, o0, m00), a01 = fmaf(-b0, o1, m01), a02 = fmaf(-b0, o2, m02);
     const float a11 = fmaf(-b1, o1, m11), a12 = fmaf(-b1, o2, m12), a22 = fmaf(-b2, o2, m22);
     const float k0 = fmaf(-vb, o0, c0), k1 = fmaf(-vb, o1, c1), k2 = fmaf(-vb, o2, c2);
-    const float r0 = a00 > thr ? rcp_ftz(a00) : 0.f;
+    const float r0 = a00 > thr ? recip(a00) : 0.f;
     const float l1 = a01 * r0, l2 = a02 * r0;
     const float d1 = fmaf(-l1, a01, a11), e1 = fmaf(-l1, a02, a12);
     const float k1p = fmaf(-l1, k0, k1), b1p = fmaf(-l1, b0, b1);
-    const float r1 = d1 > thr ? rcp_ftz(d1) : 0.f;
+    const float r1 = d1 > thr ? recip(d1) : 0.f;
     const float l3 = e1 * r1;
     const float d2 = fmaf(-l3, e1, fmaf(-l2, a02, a22));
     const float k2p = fmaf(-l3, k1p, fmaf(-l2, k0, k2)), b2p = fmaf(-l3, b1p, fmaf(-l2, b0, b2));
-    const float r2 = d2 > thr ? rcp_ftz(d2) : 0.f;
+    const float r2 = d2 > thr ? recip(d2) : 0.f;
     const float g = fmaf(k0 * b0, r0, fmaf(k1p * b1p, r1, (k2p * b2p) * r2));
     return (uc + vb) - g;
 }
 
 // S: per voxel the weighted hyperplane fit over the in-volume 3 x 3 x 3
-// neighbourhood, weights exp(-(scale v)^2).  Bound by instruction issue: 25 new
-// exponentials, about 300 instructions per voxel (the eigen-decomposition this
-// elimination replaced took 1000 more).
+// neighbourhood, weights exp(-(scale v)^2).  Bound by instruction issue: 26
+// exponentials of four instructions and about 490 instructions in all per voxel (256^3: 257 us;
+// 825 us with the eigen-decomposition that this elimination replaced).
 template <bool EDGE>
 __device__ __forceinline__ void smooth_column(float (&A)[2][SN], const float* __restrict__ u, int d, int h, int w,
                                               float ks, float* __restrict__ out, int z0, int z1, int x0, int y0) {
@@ -354,7 +344,7 @@ __global__ void __launch_bounds__(16 * DY) k_vol_pm_c(const float* __restrict__ 
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             const float gx = 0.5f * (r[k + 2] - r[k]), gy = 0.5f * (ss[k] - nn[k]), gz = 0.5f * (un[k] - ub[k]);
-            o[k] = rcp_ftz(fmaf(fmaf(gz, gz, fmaf(gx, gx, gy * gy)), ik2, 1.f));
+            o[k] = recip_ge1(fmaf(fmaf(gz, gz, fmaf(gx, gx, gy * gy)), ik2, 1.f));
             ub[k] = uc[k];
             uc[k] = un[k];
         }
@@ -428,7 +418,7 @@ cudaError_t launch_vol_quad(const float* ut, int d1, int h1, int w1, float* out,
 cudaError_t launch_vol_smooth(const float* u, int d, int h, int w, float scale, float* out, cudaStream_t s) {
     const dim3 g(blocks(w, SX), blocks(h, SY));
     const int zc = slices_per_block(d, (long long)g.x * g.y, 4);
-    k_vol_smooth<<<dim3(g.x, g.y, blocks(d, zc)), SX * SY, 0, s>>>(u, d, h, w, scale * 1.2011224087864498f, out, zc);
+    k_vol_smooth<<<dim3(g.x, g.y, blocks(d, zc)), SX * SY, 0, s>>>(u, d, h, w, scale * SQRT_LOG2E, out, zc);
     return cudaGetLastError();
 }
 
