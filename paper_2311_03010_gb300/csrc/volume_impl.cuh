@@ -380,6 +380,25 @@ __device__ __forceinline__ void sep_phase(const VolJob& J, const float* __restri
     wait_copies<0>();
 }
 
+// Four outputs from the tap list, in global memory: what rows of taps sum to where
+// every voxel is finite.  A row's taps of weight zero would carry an infinite or NaN voxel
+// (0 x inf) to outputs that no tap takes it to, so those outputs come from here.
+template <int R>
+__device__ __noinline__ float4 tap_sums(const VolJob& J, const float* __restrict__ x, int z, int y, int x0, int nv) {
+    float o[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int k = 0; k < J.taps.ntap; ++k) {
+        const int4 t = __ldg(J.gtaps + k);
+        const int gz = z + t.x, gy = y + t.y;
+        if (gz < 0 || gz >= J.d || gy < 0 || gy >= J.h) continue;
+        const float* row = x + ((long long)gz * J.h + gy) * J.w;
+        for (int i = 0; i < nv; ++i) {
+            const int gx = x0 + i + t.z;
+            if (gx >= 0 && gx < J.w) o[i] = fmaf(__int_as_float(t.w), __ldcg(row + gx), o[i]);
+        }
+    }
+    return make_float4(o[0], o[1], o[2], o[3]);
+}
+
 // One convolution phase of a PSF with dense rows of taps.
 template <int R>
 __device__ __forceinline__ void dense_phase(const VolJob& J, const float* __restrict__ x, float* sm, const EpiArgs& E,
@@ -473,7 +492,11 @@ __device__ __forceinline__ void dense_phase(const VolJob& J, const float* __rest
                     }
                 }
             }
-            if (emit) epilogue4(E, at, nv, vec, part[0], pa, pb, acc);
+            if (emit) {
+                const float4 t = part[0];
+                if (!isfinite((t.x + t.y) + (t.z + t.w))) part[0] = tap_sums<R>(J, x, z, gy, gx, nv);
+                epilogue4(E, at, nv, vec, part[0], pa, pb, acc);
+            }
 #pragma unroll
             for (int k = 0; k < 2 * R; ++k) part[k] = part[k + 1];
             part[2 * R] = make_float4(0.f, 0.f, 0.f, 0.f);
