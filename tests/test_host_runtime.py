@@ -1,0 +1,68 @@
+"""Host code against a CUDA runtime that is not there: the library's own objects linked with
+fake_cudart.cpp, which keeps a kernel's attributes per device, refuses calls on demand and
+records the launches.  No GPU is used."""
+import os
+import subprocess
+
+import pytest
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.fixture(scope="module")
+def build(tmp_path_factory):
+    from paper_2311_03010_gb300 import build_lib
+
+    build_lib.build()
+    d = tmp_path_factory.mktemp("host")
+    cuda = os.path.join(os.path.dirname(os.path.dirname(build_lib._nvcc())), "include")
+    if not os.path.isdir(cuda):
+        cuda = "/usr/local/cuda/include"
+    fake = str(d / "fake.o")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-I", cuda, "-c", os.path.join(HERE, "fake_cudart.cpp"), "-o", fake], check=True)
+
+    def run(name, source, objects):
+        src, obj, exe = (str(d / (name + e)) for e in (".cu", ".o", ""))
+        with open(src, "w") as f:
+            f.write('#include <cstdio>\n#include <cstdlib>\n#include "fake_cudart.h"\n'
+                    '#define CHECK(x) do { if (!(x)) { std::printf("line %d: %s\\n", __LINE__, #x); std::exit(1); } } while (0)\n' + source)
+        subprocess.run([build_lib._nvcc()] + build_lib.ARCH + ["-std=c++17", "--expt-relaxed-constexpr", "-I", HERE, "-I", build_lib.CSRC,
+                                                              "-c", src, "-o", obj], check=True)
+        subprocess.run(["g++", obj, fake] + [os.path.join(build_lib.BUILD, o + ".cu.o") for o in objects] + ["-o", exe], check=True)
+        r = subprocess.run([exe], capture_output=True, text=True)
+        assert r.returncode == 0, r.stdout + r.stderr
+
+    return run
+
+
+def test_large_tiles_on_a_second_device_and_after_a_refusal(build):
+    build("wide", r'''
+#include "launch.hpp"
+using namespace eecmg;
+static std::string apply(int device) {
+    fake.device = device;
+    fake.launched.clear();
+    float x = 0, y = 0;
+    Taps t{};
+    ConvArgs a;
+    a.x = &x;
+    a.y = &y;
+    a.taps = &t;
+    a.h = 900;
+    a.w = 2280;
+    for (int r = 0; r <= EECMG_MAX_RADIUS; ++r) CHECK(launch_conv(a, r, 1, 0, nullptr) == cudaSuccess);
+    CHECK(fake.launched.size() == EECMG_MAX_RADIUS + 1);
+    for (auto& n : fake.launched) CHECK((n.find("k_conv_wide") != n.npos) == (fake.launched[0].find("k_conv_wide") != n.npos));
+    return fake.launched[0];
+}
+int main() {
+    CHECK(apply(0).find("k_conv_wide") != std::string::npos);
+    CHECK(apply(1).find("k_conv_wide") != std::string::npos);
+    fake.refuse_attributes = true;  // the small tiles need none
+    CHECK(apply(2).find("k_conv_wide") == std::string::npos);
+    CHECK(cudaGetLastError() == cudaSuccess);
+    fake.refuse_attributes = false;
+    CHECK(apply(2).find("k_conv_wide") != std::string::npos);
+    return 0;
+}
+''', ["conv"])
