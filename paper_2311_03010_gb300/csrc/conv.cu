@@ -149,14 +149,15 @@ static cudaError_t launch_conv_r(const ConvArgs& a, int sep, int prec, cudaStrea
     // 23.7 -> 22.7 us; 1024^2, 171 tiles, would leave SMs idle)
     const int tiles = ((a.w + WIDE_W - 1) / WIDE_W) * ((a.h + WIDE_H - 1) / WIDE_H);
     if (a.mode == CM_STORE && sep && !prec && !a.zero_input && a.sc == nullptr && (a.w & 3) == 0 && tiles >= 304) {
-        // the attribute belongs to the current device: set for each launch (0.6 us on the
-        // host), with the small tiles where it is refused
-        if (cudaFuncSetAttribute(k_conv_wide<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Wide<R>::bytes) ==
-            cudaSuccess) {
+        // 54-78 KB of shared memory; where a device refuses them, the small tiles
+        static OncePerDevice attrs;
+        if (attrs([] {
+                return cudaFuncSetAttribute(k_conv_wide<R>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                            (int)Wide<R>::bytes) == cudaSuccess;
+            })) {
             k_conv_wide<R><<<tiles, NTHREADS, Wide<R>::bytes, s>>>(a);
             return cudaGetLastError();
         }
-        cudaGetLastError();
     }
     dim3 grid((a.w + CONV_TW - 1) / CONV_TW, (a.h + CONV_TH - 1) / CONV_TH);
     if (sep && prec)

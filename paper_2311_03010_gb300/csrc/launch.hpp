@@ -1,11 +1,34 @@
 // launch.hpp -- host-side launchers of the EECMG kernels (internal).
 #pragma once
 
+#include <atomic>
+
 #include <cuda_runtime.h>
 
 #include "common.cuh"
 
 namespace eecmg {
+
+// Sets a kernel's attributes, which belong to a device, on each device that uses it: set()
+// (true on success) runs on a device's first call, and again after a failure.
+class OncePerDevice {
+public:
+    template <class F>
+    bool operator()(F&& set) {
+        int d = 0;
+        const bool known = cudaGetDevice(&d) == cudaSuccess && d < 64;
+        if (known && (done_.load(std::memory_order_acquire) >> d & 1u)) return true;
+        if (!set()) {
+            cudaGetLastError();
+            return false;
+        }
+        if (known) done_.fetch_or(1ull << d, std::memory_order_release);
+        return true;
+    }
+
+private:
+    std::atomic<unsigned long long> done_{0};
+};
 
 // Epilogues fused into the convolution y = C (*) x.
 enum ConvMode : int {

@@ -659,13 +659,15 @@ inline int coresident_blocks(K kernel) {
     return per_sm * sms;
 }
 
+template <class K>
+inline bool wide_clusters(K kernel, OncePerDevice& attrs) {  // clusters of more than 8 blocks
+    return attrs([&] { return cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess; });
+}
+
 // Largest cluster (<= CLUSTER_MAX) the kernel can run as; 0 if none.
 template <class K>
-inline int max_cluster(K kernel) {
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess) {
-        cudaGetLastError();
-        return 0;
-    }
+inline int max_cluster(K kernel, OncePerDevice& attrs) {
+    if (!wide_clusters(kernel, attrs)) return 0;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(CLUSTER_MAX);
     cfg.blockDim = dim3(NTHREADS);
@@ -681,21 +683,22 @@ inline int max_cluster(K kernel) {
 // cluster launch of `blocks` blocks in clusters of L.cluster, or a query
 // (*out = co-resident capacity, or the largest usable cluster).
 template <class K>
-inline cudaError_t level_op(K kern, int& cap, int& cmax, const LevelLaunch& L, int op, int blocks,
-                            cudaStream_t s, int* out) {
+inline cudaError_t level_op(K kern, int& cap, int& cmax, OncePerDevice& attrs, const LevelLaunch& L, int op,
+                            int blocks, cudaStream_t s, int* out) {
     switch (op) {
         case LS_CAPACITY:
             if (cap < 0) cap = coresident_blocks(kern);
             if (out) *out = cap;
             return cudaSuccess;
         case LS_CLUSTER_MAX:
-            if (cmax < 0) cmax = max_cluster(kern);
+            if (cmax < 0) cmax = max_cluster(kern, attrs);
             if (out) *out = cmax;
             return cudaSuccess;
         case LS_COOP:
             return coop_launch(kern, L, blocks, s);
         case LS_CLUSTER:
-            if (cmax < 0) cmax = max_cluster(kern);
+            if (!wide_clusters(kern, attrs)) return cudaErrorInvalidValue;
+            if (cmax < 0) cmax = max_cluster(kern, attrs);
             if (L.cluster < 1 || L.cluster > cmax || blocks % L.cluster) return cudaErrorInvalidValue;
             return cluster_launch(kern, L, blocks, s);
         default:
@@ -707,18 +710,16 @@ inline cudaError_t level_op(K kern, int& cap, int& cmax, const LevelLaunch& L, i
 // res_smem_bytes(L.resident) of dynamic shared memory, or the largest cluster
 // it can run as with that much (cached per tile count).
 template <class K>
-inline bool res_attrs(K kern) {
-    const bool ok = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)res_smem_bytes(RES_TMAX)) == cudaSuccess &&
-                    cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
-                        cudaSuccess;
-    if (!ok) cudaGetLastError();
-    return ok;
+inline bool res_attrs(K kern, OncePerDevice& attrs) {
+    return attrs([&] {
+        return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)res_smem_bytes(RES_TMAX)) ==
+                   cudaSuccess &&
+               cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess;
+    });
 }
 
-// attrs: res_attrs() of this kernel (set once per instantiation by the caller)
 template <class K>
-inline cudaError_t res_op(K kern, bool attrs, int (&cmax)[RES_TMAX + 1], const LevelLaunch& L, int op,
+inline cudaError_t res_op(K kern, OncePerDevice& attrs, int (&cmax)[RES_TMAX + 1], const LevelLaunch& L, int op,
                           int blocks, cudaStream_t s, int* out) {
     const int T = L.resident;
     if (T < 1 || T > RES_TMAX) return cudaErrorInvalidValue;
@@ -730,7 +731,7 @@ inline cudaError_t res_op(K kern, bool attrs, int (&cmax)[RES_TMAX + 1], const L
         if (cmax[T] < 0) {
             int c = 0;
             cfg.gridDim = dim3(CLUSTER_MAX);
-            if (!attrs || cudaOccupancyMaxPotentialClusterSize(&c, kern, &cfg) != cudaSuccess) {
+            if (!res_attrs(kern, attrs) || cudaOccupancyMaxPotentialClusterSize(&c, kern, &cfg) != cudaSuccess) {
                 cudaGetLastError();
                 c = 0;
             }
@@ -739,7 +740,7 @@ inline cudaError_t res_op(K kern, bool attrs, int (&cmax)[RES_TMAX + 1], const L
         if (out) *out = cmax[T];
         return cudaSuccess;
     }
-    if (!attrs || L.cluster < 1 || L.cluster > CLUSTER_MAX || blocks % L.cluster) return cudaErrorInvalidValue;
+    if (!res_attrs(kern, attrs) || L.cluster < 1 || L.cluster > CLUSTER_MAX || blocks % L.cluster) return cudaErrorInvalidValue;
     cfg.gridDim = dim3(blocks);
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -754,14 +755,14 @@ inline cudaError_t res_op(K kern, bool attrs, int (&cmax)[RES_TMAX + 1], const L
 template <int R, bool SEP, bool PREC, bool CGLS, typename HT>
 cudaError_t launch_level_t(const LevelLaunch& L, int op, int blocks, cudaStream_t s, int* out) {
     static int cap = -1, cmax = -1;  // per instantiation; the library runs on one GPU model
+    static OncePerDevice wide;
     if (op == LS_RESIDENT || op == LS_RESIDENT_MAX) {
         if constexpr (std::is_same<HT, float>::value && R <= RES_RMAX) {
             static int rmax[RES_TMAX + 1] = {-1, -1, -1};
+            static OncePerDevice attrs;  // per instantiation
             if constexpr (CGLS) {
-                static const bool attrs = res_attrs(k_level_cgls_res<R, SEP, PREC>);  // per instantiation
                 return res_op(k_level_cgls_res<R, SEP, PREC>, attrs, rmax, L, op, blocks, s, out);
             } else {
-                static const bool attrs = res_attrs(k_level_mr2_res<R, SEP, PREC>);
                 return res_op(k_level_mr2_res<R, SEP, PREC>, attrs, rmax, L, op, blocks, s, out);
             }
         } else {
@@ -770,9 +771,9 @@ cudaError_t launch_level_t(const LevelLaunch& L, int op, int blocks, cudaStream_
         }
     }
     if constexpr (CGLS)
-        return level_op(k_level_cgls<R, SEP, PREC, HT>, cap, cmax, L, op, blocks, s, out);
+        return level_op(k_level_cgls<R, SEP, PREC, HT>, cap, cmax, wide, L, op, blocks, s, out);
     else
-        return level_op(k_level_mr2<R, SEP, PREC, HT>, cap, cmax, L, op, blocks, s, out);
+        return level_op(k_level_mr2<R, SEP, PREC, HT>, cap, cmax, wide, L, op, blocks, s, out);
 }
 
 template <int R, bool CGLS, typename HT>

@@ -66,3 +66,34 @@ int main() {
     return 0;
 }
 ''', ["conv"])
+
+
+def test_clusters_on_a_second_device_and_after_a_refusal(build):
+    build("clusters", r'''
+#include "level_solve.hpp"
+namespace eecmg {
+cudaError_t launch_level_cgls_f32_lo(const LevelLaunch& L, int rt, int sep, int prec, int op, int blocks, cudaStream_t s, int* out);
+}
+using namespace eecmg;
+static cudaError_t solve(int device, int op) {  // 16 blocks to a cluster, two tiles each where resident
+    fake.device = device;
+    fake.launched.clear();
+    LevelLaunch L;
+    L.cluster = 16;
+    L.resident = op == LS_RESIDENT ? 2 : 0;
+    const cudaError_t e = launch_level_cgls_f32_lo(L, 3, 1, 0, op, 16, nullptr, nullptr);
+    cudaGetLastError();
+    CHECK((fake.launched.size() == 1) == (e == cudaSuccess));
+    return e;
+}
+int main() {
+    for (int op : {LS_RESIDENT, LS_CLUSTER}) {
+        for (int device : {0, 1, 0}) CHECK(solve(device, op) == cudaSuccess);
+        fake.refuse_attributes = true;
+        CHECK(solve(2, op) != cudaSuccess);
+        fake.refuse_attributes = false;  // a refusal is not remembered
+        CHECK(solve(2, op) == cudaSuccess);
+    }
+    return 0;
+}
+''', ["ls_cgls_f32_lo"])
