@@ -118,58 +118,6 @@ eecmg_status plan_waves(const std::vector<std::pair<eecmg_plan_s*, int>>& items,
     return EECMG_OK;
 }
 
-cudaError_t Fan::add(int i) {
-    if (side[i]) return cudaSuccess;
-    cudaError_t e = join[i] ? cudaSuccess : cudaEventCreateWithFlags(&join[i], cudaEventDisableTiming);
-    return e == cudaSuccess ? cudaStreamCreateWithFlags(&side[i], cudaStreamNonBlocking) : e;
-}
-
-cudaError_t Fan::create(int n) {
-    cudaError_t e = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);
-    for (int i = 0; i < n && i < SIDES && e == cudaSuccess; ++i) e = add(i);
-    return e;
-}
-
-void Fan::destroy() {
-    for (int i = 0; i < SIDES; ++i) {
-        if (side[i]) cudaStreamDestroy(side[i]);
-        if (join[i]) cudaEventDestroy(join[i]);
-        side[i] = nullptr;
-        join[i] = nullptr;
-    }
-    if (fork) cudaEventDestroy(fork);
-    fork = nullptr;
-}
-
-void Fan::begin(cudaStream_t s) {
-    main_ = s;
-    n_ = 0;
-    forked_ = false;
-}
-
-cudaError_t Fan::next(cudaStream_t* out) {
-    const int i = n_ % SIDES;
-    cudaError_t e = add(i);
-    if (e != cudaSuccess) return e;  // nothing forked onto it yet
-    if (!forked_) e = cudaEventRecord(fork, main_);
-    forked_ = true;
-    if (e == cudaSuccess && n_ < SIDES) e = cudaStreamWaitEvent(side[i], fork, 0);
-    ++n_;
-    *out = side[i];
-    return e;
-}
-
-cudaError_t Fan::end() {
-    cudaError_t e = cudaSuccess;
-    for (int i = 0; i < SIDES && i < n_; ++i) {
-        cudaError_t r = cudaEventRecord(join[i], side[i]);
-        if (r == cudaSuccess) r = cudaStreamWaitEvent(main_, join[i], 0);
-        if (e == cudaSuccess) e = r;
-    }
-    n_ = 0;
-    return e;
-}
-
 void add_op(std::vector<OpGroup>& groups, size_t gi, int op, OpItem it) {
     if (groups.size() <= gi) groups.resize(gi + 1);
     groups[gi].op = op;
@@ -513,7 +461,7 @@ eecmg_status build_ctx(BatchCtx& C) {
             for (const Wave& w : C.steps[1]) k += w.cluster > 0;
         sides = std::max(sides, k);
     }
-    if (C.fan.create((int)std::min<size_t>(sides, Fan::SIDES)) != cudaSuccess) return set_error(EECMG_ERR_CUDA, "eecmg_restore_batched: side streams");
+    C.fan.create((int)std::min<size_t>(sides, Fan::SIDES));
     return EECMG_OK;
 }
 

@@ -5,6 +5,7 @@
 #include <utility>
 #include <vector>
 
+#include "fan.hpp"
 #include "launch.hpp"
 #include "level_solve.hpp"
 #include "plan.hpp"
@@ -33,32 +34,6 @@ LevelJob make_job(eecmg_plan_s* P, int l);
 // out in a fixed order (by cluster size and instantiation, then item order).
 eecmg_status plan_waves(const std::vector<std::pair<eecmg_plan_s*, int>>& items,
                         std::vector<HostWave>& waves);
-
-// Side streams on which the cluster-mode waves of a step run beside its cooperative
-// ones.  Every wave of a step works on images of its own, so the order between
-// them is free.  A cluster is scheduled whole and waits for no other launch, so
-// cluster waves may overlap each other and a cooperative wave; cooperative waves
-// stay in one chain, since two of them may not be resident together.  24 uneven
-// images launch up to 13 cluster waves a step, each a few blocks for 30-70 us.
-struct Fan {
-    static constexpr int SIDES = 8;
-    cudaStream_t side[SIDES] = {};
-    cudaEvent_t fork = nullptr, join[SIDES] = {};
-    // n side streams at once (a capture creates none); further ones come at first use
-    cudaError_t create(int n);
-    void destroy();
-    // Queues a cluster launch on the next side stream; begin() forks the side streams
-    // off s at their first use, end() joins those used back into s.
-    void begin(cudaStream_t s);
-    cudaError_t next(cudaStream_t* out);
-    cudaError_t end();
-
-private:
-    cudaError_t add(int i);
-    cudaStream_t main_ = nullptr;
-    int n_ = 0;       // cluster launches so far
-    bool forked_ = false;
-};
 
 // Per-level operations of many images, one launch per group (a group holds
 // one kind of operation, k_ops_batch).

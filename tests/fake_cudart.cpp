@@ -89,6 +89,32 @@ cudaError_t cudaFuncSetAttribute(const void* f, cudaFuncAttribute a, int v) {
     if (a == cudaFuncAttributeNonPortableClusterSizeAllowed) x.wide_clusters = v != 0;
     return cudaSuccess;
 }
+cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned int) {
+    static char* next = nullptr;
+    if (fake.streams_left <= 0) return result(cudaErrorMemoryAllocation);
+    --fake.streams_left;
+    ++fake.made;
+    *s = (cudaStream_t)(next += 16);
+    return cudaSuccess;
+}
+cudaError_t cudaStreamDestroy(cudaStream_t) {
+    --fake.made;
+    return cudaSuccess;
+}
+cudaError_t cudaEventCreateWithFlags(cudaEvent_t* e, unsigned int) {
+    ++fake.made;
+    *e = (cudaEvent_t)&fake;
+    return cudaSuccess;
+}
+cudaError_t cudaEventDestroy(cudaEvent_t) {
+    --fake.made;
+    return cudaSuccess;
+}
+cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaStreamWaitEvent(cudaStream_t s, cudaEvent_t, unsigned int) {
+    fake.waits.push_back(s);
+    return cudaSuccess;
+}
 cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void**) {
     unsigned int cluster = 1;
     for (unsigned int i = 0; i < c->numAttrs; ++i)

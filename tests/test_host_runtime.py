@@ -28,7 +28,7 @@ def build(tmp_path_factory):
                     '#define CHECK(x) do { if (!(x)) { std::printf("line %d: %s\\n", __LINE__, #x); std::exit(1); } } while (0)\n' + source)
         subprocess.run([build_lib._nvcc()] + build_lib.ARCH + ["-std=c++17", "--expt-relaxed-constexpr", "-I", HERE, "-I", build_lib.CSRC,
                                                               "-c", src, "-o", obj], check=True)
-        subprocess.run(["g++", obj, fake] + [os.path.join(build_lib.BUILD, o + ".cu.o") for o in objects] + ["-o", exe], check=True)
+        subprocess.run(["g++", obj, fake] + [os.path.join(build_lib.BUILD, o + ".o") for o in objects] + ["-o", exe], check=True)
         r = subprocess.run([exe], capture_output=True, text=True)
         assert r.returncode == 0, r.stdout + r.stderr
 
@@ -65,7 +65,7 @@ int main() {
     CHECK(apply(2).find("k_conv_wide") != std::string::npos);
     return 0;
 }
-''', ["conv"])
+''', ["conv.cu"])
 
 
 def test_clusters_on_a_second_device_and_after_a_refusal(build):
@@ -96,4 +96,46 @@ int main() {
     }
     return 0;
 }
-''', ["ls_cgls_f32_lo"])
+''', ["ls_cgls_f32_lo.cu"])
+
+
+def test_side_streams_are_made_once_and_done_without(build):
+    build("fan", r'''
+#include <set>
+#include "fan.hpp"
+using namespace eecmg;
+static std::vector<cudaStream_t> waves(Fan& f, cudaStream_t s, int n) {
+    std::vector<cudaStream_t> got(n);
+    fake.waits.clear();
+    f.begin(s);
+    for (auto& t : got) CHECK(f.next(&t) == cudaSuccess);
+    CHECK(f.end() == cudaSuccess);
+    return got;
+}
+int main() {
+    cudaStream_t s = (cudaStream_t)0x1000;
+    for (int want : {0, 1, 3, Fan::SIDES}) {
+        for (int limit : {0, 1, 2, 100}) {  // streams that can be made
+            Fan f;
+            fake.streams_left = limit;
+            f.create(want);
+            CHECK(cudaGetLastError() == cudaSuccess);
+            const int made = fake.made;
+            const int sides = want < limit ? want : limit;
+            for (int n : {0, 1, 2, 5, 20}) {
+                const auto got = waves(f, s, n);
+                const std::set<cudaStream_t> used(got.begin(), got.end());
+                CHECK((int)used.size() == (sides == 0 ? (n > 0) : n < sides ? n : sides));
+                if (sides == 0) CHECK(n == 0 || *used.begin() == s);
+                // every side stream used waits for the main one, and the main one for each
+                CHECK(fake.waits.size() == (sides == 0 ? 0 : 2 * used.size()));
+                for (size_t i = 0; i < fake.waits.size(); ++i) CHECK((fake.waits[i] == s) == (i >= used.size()));
+            }
+            CHECK(fake.made == made);  // nothing made after create()
+            f.destroy();
+            CHECK(fake.made == 0);
+        }
+    }
+    return 0;
+}
+''', ["fan.cpp"])
