@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(NTHREADS) k_conv(ConvArgs a) {
 }
 
 // y = C (*) x alone (CM_STORE), separable, on the large tiles of conv_wide.cuh, one per
-// block: 3 blocks per SM overlap one another's copies and passes.
+// block: 3 blocks per SM (2 from r = 11 on) overlap one another's copies and passes.
 template <int R>
 __global__ void __launch_bounds__(NTHREADS, 2) k_conv_wide(ConvArgs a) {
     extern __shared__ float4 wide_smem[];
@@ -130,8 +130,8 @@ __global__ void __launch_bounds__(NTHREADS, 2) k_conv_wide(ConvArgs a) {
     }
     float* y = a.y;
     const bool vec = (reinterpret_cast<uintptr_t>(y) & 15) == 0;
-    wide_conv<R>(reinterpret_cast<float*>(wide_smem), taps, taps + 2 * R + 1, a.x, a.h, a.w, gridDim.x, blockIdx.x,
-                 nullptr, [&](size_t i, float4 z, float4) {
+    wide_conv<R>(reinterpret_cast<float*>(wide_smem), taps, taps + 2 * R + 1, a.x, a.h, a.w, blockIdx.x,
+                 [&](size_t i, float4 z) {
                      if (vec) {
                          st4(y, i >> 2, z);
                      } else {

@@ -1,7 +1,7 @@
 // conv_wide.cuh -- the separable convolution on large tiles, 56 x 120 outputs, for
 // one application of H to a large image.
 //
-// GB300, 2160 x 3840, r = 6: 32.8 -> 26.7 us; 4096^2, r = 10: 70 -> 60 us (66 MB and
+// GB300, 2160 x 3840, r = 6: 32.8 -> 26.3 us; 4096^2, r = 10: 70 -> 60 us (66 MB and
 // 134 MB would take 10 and 20 us; issue slots are two thirds busy).  The level
 // solvers keep the 32 x 64 tiles: with these, a 4096^2 solve was as fast (367 us
 // against 367 at r = 10, 340 against 325 at r = 6), a 2048^2 one slower (149 against
@@ -12,9 +12,10 @@
 // four barriers per 2048 pixels.  Here a thread of the vertical pass owns four
 // columns of 8 rows (28 16-byte loads for 32 outputs; 36 quads x 7 groups keep 252
 // of 256 threads busy at the largest radius), the horizontal pass owns four
-// columns of a row and stores them itself, and the next tile's window arrives by
-// cp.async while it runs: two barriers per 6720 pixels.  Each output sums its taps
-// in increasing order, vertical pass first, as in conv_tile.cuh (the same value).
+// columns of a row and stores them itself: two barriers per 6720 pixels.  A block
+// takes one tile; the other blocks of its SM run while its window arrives by cp.async.
+// Each output sums its taps in increasing order, vertical pass first, as in
+// conv_tile.cuh (the same value).
 #pragma once
 
 #include "launch.hpp"
@@ -77,64 +78,51 @@ __device__ __forceinline__ void wide_vertical(const float* A, float* tmp, const 
     for (int i = 0; i < W::VR; ++i) t[i * W::QX] = acc[i];
 }
 
-// One convolution over the level's tiles bid, bid + nb, ...: epi(index, (C (*) x) of
-// four pixels, pre of them); w a multiple of 4.  sm: Wide<R>::bytes; cy, cx: the taps
-// centred at R in shared memory.  Called by all threads of the block.
+// The convolution of tile t: epi(index, (C (*) x) of four pixels); w a multiple of 4.
+// sm: Wide<R>::bytes; cy, cx: the taps centred at R in shared memory.  Called by all
+// threads of the block.
 template <int R, class Epi>
 __device__ __forceinline__ void wide_conv(float* sm, const float* cy, const float* cx, const float* x, int h, int w,
-                                          unsigned int nb, unsigned int bid, const float* pre, Epi&& epi) {
+                                          int t, Epi&& epi) {
     using W = Wide<R>;
     float* A = sm;
     float* tmp = sm + W::IN;
-    const int tx = (w + W::WW - 1) / W::WW, ntiles = tx * ((h + W::WH - 1) / W::WH);
-    const bool vec = (reinterpret_cast<uintptr_t>(x) & 15) == 0, pvec = (reinterpret_cast<uintptr_t>(pre) & 15) == 0;
-    __syncthreads();  // the caller's use of sm and the taps
-    if ((int)bid < ntiles) wide_stage<R>(x, h, w, ((int)bid / tx) * W::WH, ((int)bid % tx) * W::WW, A, vec);
+    const int tx = (w + W::WW - 1) / W::WW, y0 = (t / tx) * W::WH, x0 = (t % tx) * W::WW;
+    wide_stage<R>(x, h, w, y0, x0, A, (reinterpret_cast<uintptr_t>(x) & 15) == 0);
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();  // the window and the taps
+    wide_vertical<R>(A, tmp, cy);
+    __syncthreads();
+    float c[W::NT];
+#pragma unroll
+    for (int d = 0; d < W::NT; ++d) c[d] = cx[d];
 #pragma unroll 1
-    for (int t = (int)bid; t < ntiles; t += (int)nb) {
-        const int y0 = (t / tx) * W::WH, x0 = (t % tx) * W::WW;
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
-        __syncthreads();
-        wide_vertical<R>(A, tmp, cy);
-        __syncthreads();
-        const int tn = t + (int)nb;
-        if (tn < ntiles) wide_stage<R>(x, h, w, (tn / tx) * W::WH, (tn % tx) * W::WW, A, vec);
-        float c[W::NT];
+    for (int i = threadIdx.x; i < W::WH * (W::WW / 4); i += NTHREADS) {
+        const int r = i / (W::WW / 4), q = i - r * (W::WW / 4);
+        const int gy = y0 + r, gx = x0 + 4 * q;
+        if (gy >= h || gx >= w) continue;
+        constexpr int NQ = 1 + 2 * W::PADX / 4;
+        const float4* s = reinterpret_cast<const float4*>(tmp) + r * W::QX + q;
+        float v[4 * NQ];
 #pragma unroll
-        for (int d = 0; d < W::NT; ++d) c[d] = cx[d];
-#pragma unroll 1
-        for (int i = threadIdx.x; i < W::WH * (W::WW / 4); i += NTHREADS) {
-            const int r = i / (W::WW / 4), q = i - r * (W::WW / 4);
-            const int gy = y0 + r, gx = x0 + 4 * q;
-            if (gy >= h || gx >= w) continue;
-            const size_t idx = (size_t)gy * w + gx;
-            float4 p = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (pre) p = pvec ? __ldcg(reinterpret_cast<const float4*>(pre + idx))
-                              : make_float4(__ldcg(pre + idx), __ldcg(pre + idx + 1), __ldcg(pre + idx + 2), __ldcg(pre + idx + 3));
-            constexpr int NQ = 1 + 2 * W::PADX / 4;
-            const float4* s = reinterpret_cast<const float4*>(tmp) + r * W::QX + q;
-            float v[4 * NQ];
-#pragma unroll
-            for (int j = 0; j < NQ; ++j) {
-                const float4 u = s[j];
-                v[4 * j] = u.x;
-                v[4 * j + 1] = u.y;
-                v[4 * j + 2] = u.z;
-                v[4 * j + 3] = u.w;
-            }
-            float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-            for (int d = 0; d < W::NT; ++d) {
-                constexpr int b = W::PADX - R;
-                o.x = fmaf(c[d], v[b + d], o.x);
-                o.y = fmaf(c[d], v[b + d + 1], o.y);
-                o.z = fmaf(c[d], v[b + d + 2], o.z);
-                o.w = fmaf(c[d], v[b + d + 3], o.w);
-            }
-            epi(idx, o, p);
+        for (int j = 0; j < NQ; ++j) {
+            const float4 u = s[j];
+            v[4 * j] = u.x;
+            v[4 * j + 1] = u.y;
+            v[4 * j + 2] = u.z;
+            v[4 * j + 3] = u.w;
         }
+        float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int d = 0; d < W::NT; ++d) {
+            constexpr int b = W::PADX - R;
+            o.x = fmaf(c[d], v[b + d], o.x);
+            o.y = fmaf(c[d], v[b + d + 1], o.y);
+            o.z = fmaf(c[d], v[b + d + 2], o.z);
+            o.w = fmaf(c[d], v[b + d + 3], o.w);
+        }
+        epi((size_t)gy * w + gx, o);
     }
-    __syncthreads();  // sm is the caller's again
 }
 
 }  // namespace eecmg
