@@ -163,14 +163,13 @@ __device__ __forceinline__ float denoise_value_rd(Ud in, Cd c, int h, int w, flo
     return pm_step(uc, fe, fw, fn, fs, tau);
 }
 // The start of a prolonged level (Algorithm 2, Step 2) in one pass: D(S(P(Pi(u1, u2)))) for
-// one TH x PSD_TW block of fine pixels at (y0, x0), TH <= PSD_TH (the shared-memory stages are
-// sized for PSD_TH rows; a block's result does not depend on TH).  D needs S's output with a 2-pixel halo
+// one PSD_TH x PSD_TW block of fine pixels at (y0, x0).  D needs S's output with a 2-pixel halo
 // (its own 4 neighbours and their diffusivities), S needs P's with a 1-pixel halo beyond that,
 // and P the level-(l-1) window of Pi values its triplets read; each stage is computed for its
 // whole region into shared memory (pixels outside the image are never read), with the
 // per-pixel arithmetic of k_prolong, k_smooth and k_denoise, so the result equals those three
 // kernels in sequence bitwise, while the two intermediate images never leave the SM.  Halo
-// work at TH = 32: P on 1.30x, S on 1.20x, c on 1.10x the block's pixels.  Called by every thread of a
+// work: P on 1.30x, S on 1.20x, c on 1.10x the block's pixels.  Called by every thread of a
 // 256-thread block; store(rr, cc, v) receives the block's in-image outputs (row rr, column cc of
 // the tile).
 constexpr int PSD_TH = 32, PSD_TW = 64, PSD_THREADS = 256;
@@ -189,13 +188,12 @@ struct PsdSmem {
     float S[PSD_SH][PSD_SW];
     float C[PSD_CH][PSD_CW];
 };
-template <int TH = PSD_TH, class Store>
+template <class Store>
 __device__ __forceinline__ void tile_psd(PsdSmem& M, const float* __restrict__ u1, int h1, int w1,
                                          const float* __restrict__ u2, int h2, int w2, int h, int w,
                                          float scale, float tau, float inv_k2, int y0, int x0,
                                          Store&& store) {
-    static_assert(TH >= 1 && TH <= PSD_TH, "the stages are sized for PSD_TH rows");
-    constexpr int th = TH;
+    constexpr int th = PSD_TH;
     const int tid = threadIdx.y * blockDim.x + threadIdx.x;
     constexpr int NT = PSD_THREADS;
     // fine region of P (clipped to the image) and its Pi window
@@ -227,7 +225,7 @@ __device__ __forceinline__ void tile_psd(PsdSmem& M, const float* __restrict__ u
         M.X[rr][cc] = pi_from(u1[(size_t)a * w1 + b], dd(A0, B0), dd(A0, B1), dd(A1, B0), dd(A1, B1));
     }
     __syncthreads();
-    // P on rows y0-3 .. y0+TH+2 and columns x0-3 .. x0+TW+2 (in-image part)
+    // P on rows y0-3 .. y0+th+2 and columns x0-3 .. x0+PSD_TW+2 (in-image part)
     for (int k = tid; k < (th + 6) * PSD_PW; k += NT) {
         const int rr = k / PSD_PW, cc = k - rr * PSD_PW;
         const int y = y0 - 3 + rr, x = x0 - 3 + cc;
