@@ -422,7 +422,11 @@ __device__ __forceinline__ float recip_ge1(float x) {
     const float r = __fmaf_rn(y, __fmaf_rn(-x, y, 1.f), y);
     return x < 0x1p126f ? r : y;
 }
-constexpr float SQRT_LOG2E = 1.2011224087864498f;  // exp(-(s v)^2) = 2^-(SQRT_LOG2E s v)^2
+// ks = scale sqrt(log2 e), so that exp(-(scale v)^2) = 2^-(ks v)^2; finite at the largest
+// scales too (between equal neighbours v = 0 and the weight is 1).
+__host__ __device__ __forceinline__ float s_scale_ks(float scale) {
+    return fabsf(scale) < 2.8e38f ? scale * 1.2011224087864498f : copysignf(3.4e38f, scale);
+}
 
 __device__ __forceinline__ float dot4(float4 a, float4 b, float acc) {
     acc = fmaf(a.x, b.x, acc);

@@ -61,9 +61,8 @@ static __constant__ float c_qw[4][3] = {
 // rounding of each operation fixed (no contraction), so that the kernels'
 // results agree bitwise: the pair terms below, and s_value.
 
-// exp(-(scale v)^2) from ks = scale sqrt(log2 e): the weight of a pair of
+// exp(-(scale v)^2) from ks = s_scale_ks(scale): the weight of a pair of
 // neighbours; it does not depend on which of the two is the centre.
-__device__ __forceinline__ float s_scale_ks(float scale) { return __fmul_rn(scale, SQRT_LOG2E); }
 __device__ __forceinline__ float s_weight(float v, float ks) {
     const float t = __fmul_rn(v, ks);
     return ex2_approx(__fmul_rn(t, -t));

@@ -418,7 +418,7 @@ cudaError_t launch_vol_quad(const float* ut, int d1, int h1, int w1, float* out,
 cudaError_t launch_vol_smooth(const float* u, int d, int h, int w, float scale, float* out, cudaStream_t s) {
     const dim3 g(blocks(w, SX), blocks(h, SY));
     const int zc = slices_per_block(d, (long long)g.x * g.y, 4);
-    k_vol_smooth<<<dim3(g.x, g.y, blocks(d, zc)), SX * SY, 0, s>>>(u, d, h, w, scale * SQRT_LOG2E, out, zc);
+    k_vol_smooth<<<dim3(g.x, g.y, blocks(d, zc)), SX * SY, 0, s>>>(u, d, h, w, s_scale_ks(scale), out, zc);
     return cudaGetLastError();
 }
 

@@ -110,3 +110,17 @@ def test_weights_below_the_normal_range_count(gpu, v):
         assert host(y)[0] == pytest.approx(want, rel=2.0 ** -11, abs=0)
     plan.close()
     vol.close()
+
+
+# The largest scales: between equal neighbours the weight is 1 and a constant stays.
+@pytest.mark.parametrize("scale", [1e38, 3e38, 3.402823e38])
+def test_a_constant_stays_at_every_scale(gpu, scale):
+    torch, E = gpu
+    x = torch.full((5, 7, 9), 5.0, device="cuda")
+    plan, vol = E.Plan(9, 35, 1, np.ones((1, 1)), s_scale=scale), E.VolumePlan(9, 7, 5, 1, np.ones((1, 1, 1)), s_scale=scale)
+    for smooth, h in ((E.eecmg_smooth, plan.handle), (E.eecmg_vol_smooth, vol.h)):
+        y = torch.empty_like(x)
+        smooth(h, 0, x, y)
+        assert torch.equal(x, y)
+    plan.close()
+    vol.close()
