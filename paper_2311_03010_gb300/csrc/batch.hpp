@@ -29,9 +29,9 @@ LevelJob make_job(eecmg_plan_s* P, int l);
 // Groups the level solves items[i] = (plan, level) into waves.  Every job
 // gets the partition of the same solve launched alone (level_shape), so each
 // result is bitwise that of the plan's own restoration.  Cluster-mode jobs of
-// one instantiation share one launch; cooperative jobs that do not fit the
-// co-resident capacity of their instantiation start a new wave.  Groups come
-// out in a fixed order (by cluster size and instantiation, then item order).
+// one instantiation share one launch; cooperative jobs go largest first into the
+// first wave with room within the co-resident capacity of their instantiation.
+// Groups come out in a fixed order (by cluster size and instantiation).
 eecmg_status plan_waves(const std::vector<std::pair<eecmg_plan_s*, int>>& items,
                         std::vector<HostWave>& waves);
 

@@ -353,11 +353,12 @@ int op_blocks_x(int op, int w) { return op == OP_PSD ? (w + ST_COLS - 1) / ST_CO
 
 // Rows per strip segment of the level starts of one launch (a segment computes
 // 6 rows more than it stores).  Where a quarter of the register file's warps
-// hold segments of MIN_ROWS, the chain of rows is the time: 9 us for a 64^2 to
-// 256^2 level in segments of 4 rows, 12 us in segments of 8.  Beyond that the
-// SMs are loaded and the extra rows count (1024^2: 17 us in 8 rows, 20 us in 4):
-// the fewest rows from psd_tile_rows() / 4 to 64 at which all segments are
-// resident at once.
+// hold segments of MIN_ROWS, the chain of rows is the time: 11 us for a 64^2 to
+// 256^2 level in segments of 4 rows, 15 us in segments of 8.  Beyond that the
+// SMs are loaded and the extra rows count (1024^2: 20.5 us in 8 rows, 22.7 us in 4):
+// the fewest rows from psd_tile_rows() / 4 on at which all segments are resident
+// at once, at most 64 (beyond 3600^2 they no longer are: 4096^2 has 2304 segments for
+// 1824 places).
 void place_starts(OpItem* items, int n) {
     constexpr long long SMS = 152, MIN_ROWS = 4, MAX_ROWS = 64;
     auto units = [&](long long th) {

@@ -1,8 +1,8 @@
 // level_start.cuh -- the start of a prolonged level (Algorithm 2, Step 2),
 // D(S(P(Pi(u1, u2)))), one warp per strip of columns marching down the rows.
 //
-// The operator chain is instruction-bound (S alone takes eight weights, a 2 x 2
-// eigen-problem and a projection per pixel), so the kernel is built to issue few
+// The operator chain is instruction-bound (S alone takes eight weights, nine moments
+// and an elimination per pixel), so the kernel is built to issue few
 // instructions per pixel and to need no barrier:
 //   - a lane owns one level-(l-2) cell: 4 fine columns, two level-(l-1) columns
 //     and one node; Pi's node differences, its double-float sums and P's column
@@ -18,8 +18,9 @@
 // k_smooth and k_denoise (bitwise), so a result does not depend on the split.
 //
 // GB300, one start (32 x 64 tiles staged in shared memory before -> this): 4096^2 312
-// -> 126 us, 2048^2 88 -> 38 us, 64^2 19 -> 9 us; its 88 MB at 4096^2 would take 13 us, so
-// it stays bound by the issue of its instructions.
+// -> 161 us, 2048^2 88 -> 49 us, 64^2 19 -> 11 us; its 88 MB at 4096^2 would take 13 us, so
+// it stays bound by the issue of its instructions (22 us of the 161 are the exponentials'
+// subnormal results, 16 the correctly rounded reciprocals).
 #pragma once
 
 #include "level_ops.cuh"

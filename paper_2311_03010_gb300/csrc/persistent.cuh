@@ -44,8 +44,8 @@ __device__ __forceinline__ unsigned int ld_acquire(const unsigned int* p) {
     return v;
 }
 
-// Every thread of every block of the job calls this with its NV FP32 values
-// in v (thread-local contributions).  partials holds 2 x nb x NPART
+// Every thread of every block of the job calls this with its NV values (thread-local
+// contributions, as pairs).  partials holds 2 x nb x NPART
 // double-float slots (8 bytes each).  All sums run in double-float on the FP32
 // pipes, and finish receives the job totals as double-float pairs.  Returns false if the
 // job is in error (the caller returns).

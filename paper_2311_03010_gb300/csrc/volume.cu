@@ -10,8 +10,8 @@
 //                differences                                         (Section 3.2)
 //   P            the three-point quadratic rule along all three axes (Section 3.2)
 //   S            weighted hyperplane fit over the 3x3x3 neighbourhood with the
-//                Eq. 18 weights, pseudo-inverse of the 3x3 moment matrix
-//                (eigenvalues under 1e-6 W dropped)                  (Section 3.3)
+//                Eq. 18 weights, elimination on the 3x3 moment matrix
+//                (pivots of at most 1e-6 W dropped)                  (Section 3.3)
 //   D            one explicit Perona-Malik step with six face neighbours
 //                                                                    (Section 4)
 //   C_l^m        MR-II with the discrepancy stop of Section 2 and m_l as its cap.
@@ -497,8 +497,8 @@ eecmg_status eecmg_vol_plan(int width, int height, int depth, int levels, const 
         return set_error(EECMG_ERR_CUDA, std::string("eecmg_vol_plan: ") + cudaGetErrorString(e));
     }
     // few slices per block to march (two blocks per SM): tiles (62 x 146 x 25, r = 3, 1.2 slices
-    // a block: solve 121 us marched, 83 us in tiles; 256^3, 33 slices a block: 46 against 113 us
-    // a convolution)
+    // a block: solve 121 us marched, 83 us in tiles; 256^3, 34 slices a block: 46 against 113 us
+    // a convolution).  SmallTile has both sides around the line.
     for (int l = 0; l < L; ++l)
         for (VolTaps* t : {&P->taps[l], &P->tapsT[l]})
             if (t->form == VF_SEP && level_units(P->ds[l], P->hs[l], P->ws[l], *t) < 2LL * t->r * 2 * P->sms)

@@ -87,7 +87,8 @@ __device__ __forceinline__ void acc_add(DF& a, float v) {
 // So a voxel costs 3 (2 r + 1) multiplications, about a quarter of a shared
 // load per multiplication and no index arithmetic beyond its row.
 // VF_DENSE: the thread's window of each row enters all 2 r + 1 slices' partial sums.
-// A range repeats the 2 r slices around its start, 2 r / 54 of the work at 256^3.
+// A range repeats the 2 r slices around its start: at 256^3 and r = 3, 6 to 34 (VF_SEP,
+// 10 x 4 tiles of 28 rows) or to 54 (VF_DENSE, 16 x 4 of 16 rows) of its own.
 // What a phase does with H x: out = H x (or a - H x) and its sums.
 enum VolEpi : int { VE_RESID = 0, VE_STORE, VE_Q1, VE_Z };
 struct EpiArgs {
@@ -564,8 +565,11 @@ __device__ __forceinline__ void sparse_phase(const VolJob& J, const float* __res
 // volume) in flight by cp.async while this one is convolved: slices over every
 // staged (row, column) into B, rows into C (over the window's own buffer),
 // columns over C.  A marching block repeats 2 r slices whatever its share, so below
-// 2 r slices a block the tiles are faster (GB300, 45 x 70 x 61, r = 2: 4.4 us a
-// convolution against 5.9 us; 128^3, 4.2 slices a block, 11.2 against 10.9 us).
+// 2 r slices a block the tiles are faster.  GB300, one convolution in tiles | marched, us:
+// 45 x 70 x 61, r = 2 (0.4 slices a block) 4.7 | 5.8; 62 x 146 x 25, r = 3 (1.2) 5.0 | 13.3; 128^3
+// (4.2 up to r = 4) r = 1 10.0 | 7.5, r = 2 11.8 | 10.8, r = 3 15.0 | 15.7, r = 4 16.0 | 21.2;
+// 160^3, r = 3 (9.5) 27.2 | 21.9.  The line was drawn up to r = 4: with the 12-row tiles
+// of r = 6 marching is ahead of it, 128^3 (9.3 slices a block) 44.1 | 28.6.
 template <int R>
 struct SmallTile {
     static constexpr int PADX = (R + 3) / 4 * 4, X0 = PADX - R;

@@ -6,9 +6,9 @@
 // A thread owns a column (Pi, P: a cell of a column) and marches along the
 // slices, so that what a slice contributes to its neighbours is formed once
 // and kept in registers; in-slice neighbours come from shared-memory planes.
-// GB300 at 256^3, one voxel per thread before -> now: Pi (128^3) 19 -> 10 us, P
-// 206 -> 17 us (its taps came from a per-lane constant index), S 825 -> 257 us, D
-// 140 -> 64 us (134 + 201 MB: at the memory's rate).
+// GB300 at 256^3, one voxel per thread before -> now: Pi (128^3) 19 -> 11 us, P
+// 206 -> 18 us (its taps came from a per-lane constant index), S 825 -> 245 us, D
+// 140 -> 70 us (134 + 201 MB: at the memory's rate).
 #include <algorithm>
 #include <cstdint>
 
@@ -183,8 +183,8 @@ __device__ __forceinline__ float fit_value(float uc, const Plane& T, const Plane
 
 // S: per voxel the weighted hyperplane fit over the in-volume 3 x 3 x 3
 // neighbourhood, weights exp(-(scale v)^2).  Bound by instruction issue: 26
-// exponentials of four instructions and about 490 instructions in all per voxel (256^3: 257 us;
-// 825 us with the eigen-decomposition that this elimination replaced).
+// exponentials of four instructions and 464 instructions in all per voxel (256^3: 245 us, issuing
+// 87 % of the time; 825 us with the eigen-decomposition that this elimination replaced).
 template <bool EDGE>
 __device__ __forceinline__ void smooth_column(float (&A)[2][SN], const float* __restrict__ u, int d, int h, int w,
                                               float ks, float* __restrict__ out, int z0, int z1, int x0, int y0) {
